@@ -119,7 +119,8 @@ int dtp_affinity_accumulate_ex(const void* X, const void* C, const void* W_gate,
  *   max_ctas   0: one persistent CTA per SM (the default of the other entry
  *              points); n > 0: at most n CTAs, leaving the other SMs to
  *              kernels running concurrently on other streams (for instance the
- *              layout search of the previous layer, which runs on one SM).
+ *              layout search of the previous layer, which runs on two SMs when the layer's
+ *              gains fit in one block's shared memory, else on up to 16).
  *              When the layer's W_gate and W_up fit in half of the L2 cache
  *              the kernel runs as pairs of CTAs, and n is then rounded down
  *              to an even count (at least one pair: 2 CTAs for n = 1)
@@ -393,7 +394,7 @@ int dtp_search_layout(const float* A, int H_kv, int N, int D, int iters,
  * dtp_search_layout on `layers` independent layers at once (the up-edge
  * objective decouples across layers); layer i reads A + i*H_kv*N and writes
  * head_part + i*H_kv, neuron_dev + i*N, score_q[i], score[i], iters_done[i].
- * One thread block per layer.  Asynchronous; the workspace status word holds
+ * One thread block or cluster of blocks per layer.  Asynchronous; the workspace status word holds
  * the most severe device-side status over the layers (DTP_ERR_NOT_CONVERGED
  * before DTP_ERR_ARG before DTP_OK).
  */

@@ -43,6 +43,14 @@ def test_chain_matches_oracle(L, G, N, D, kind):
     _compare(Su, Sd, D, 10)
 
 
+@pytest.mark.parametrize("L,G,N,D,kind", [(2, 8, 4104, 8, "lognormal"), (2, 8, 3864, 8, "integer"),
+                                          (30, 8, 1540, 4, "lognormal")])
+def test_chain_layer_splits(L, G, N, D, kind):
+    """Slices of a layer on several blocks (N = 3864 and 4104 at D = 8), and gathered on two of them."""
+    Su, Sd = _model(L, G, N, seed=L + N, kind=kind)
+    _compare(Su, Sd, D, 10)
+
+
 @pytest.mark.parametrize("iters", [1, 2])
 def test_chain_iteration_cap(iters):
     Su, Sd = _model(4, 8, 256, seed=9)

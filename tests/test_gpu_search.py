@@ -81,6 +81,16 @@ def test_full_size_qwen_d2_and_d4():
             _compare(An[i], D, 10, res={k: v[i] for k, v in res.items()}, unique=True)
 
 
+@pytest.mark.parametrize("G,N,D,kind", [
+    (8, 776, 4, "lognormal"), (8, 1544, 4, "lognormal"), (6, 9000, 3, "integer"),   # one block and two, a gathered layer
+    (8, 4096, 8, "integer"), (8, 4096, 8, "lognormal"), (4, 16400, 4, "lognormal"),  # slices on several blocks
+    (2, 262144, 2, "lognormal")])                                                    # gains in global memory
+def test_search_layer_splits(G, N, D, kind):
+    """How a layer is spread over blocks: sizes on both sides of each line, with and without ties."""
+    A = synth.make_affinity_matrix(G, N, seed=G + N + D, kind=kind).numpy()
+    _compare(A, D, 10)
+
+
 def test_full_size_llama_neuron_count_d8():
     """Llama-3.1-8B shape N=14336 (global-memory path of the search), D=8."""
     A = synth.make_affinity_matrix(8, 14336, seed=3).numpy()
