@@ -2,11 +2,12 @@
 // scores") on the CUDA cores, plus the finalize and ||w^d||^2 helpers.
 //
 // The fp32 mode exists for tight checks (fp32 operands, fp32 FMA); TF32
-// tensor cores would not meet a 1e-5 relative error.  A block computes a
-// 64-token x 64-neuron tile: the X pass gives (alpha, beta) per (token, neuron)
-// in registers, then each head pass gives (pg, pu) and Delta^2 is summed over
-// the block's tokens.  Per-tile partials go to the workspace and are added
-// into A in a fixed order, so the result is deterministic.
+// tensor cores would not meet a 1e-5 relative error.  A block computes a tile
+// of 128 x 128 (or 64 x 64) tokens and neurons, gate and up together: the X pass gives
+// (alpha, beta) per (token, neuron), kept in shared memory, then each head pass
+// gives (pg, pu) and Delta^2 is summed over the block's tokens.  Per-tile
+// partials go to the workspace and are added into A in a fixed order, so the
+// result is deterministic.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -16,124 +17,217 @@
 namespace dtp {
 namespace f32 {
 
-constexpr int TT = 64;   // tokens per tile
-constexpr int TN = 64;   // neurons per tile
-constexpr int TK = 16;   // k chunk
+constexpr int TK = 16;        // k block
 constexpr int kThreads = 256;
+constexpr int kTokMin = 64;   // tokens per tile of the smaller form (the workspace is sized for it)
 
-// acc_g[i][j] = sum_k act[t_i,k] Wg[n_j,k], acc_u likewise, for the thread's
-// tokens t_i = t0 + ty + 16 i and neurons n_j = n0 + tx + 16 j.
+// Bound by the FMA pipe.  A thread owns TPT tokens x NPT neurons of gate and of up and multiplies with
+// packed fma.rn.f32x2 (each half rounds as a scalar fma: the sums over k are those of a scalar loop), a
+// weight pair from shared memory times an activation repeated in both halves.  8 x 8 per thread (128 x 128
+// tiles, one block per SM): per k six float4 shared loads for 64 packed FMAs, which keeps the pipe and not
+// the loads the limit; 4 x 4 (64 x 64 tiles, two blocks per SM) for layers with few tiles.  alpha and beta
+// live in shared memory, the next k block is loaded from global memory during the current one.
+// T = 1024, d = 1024, 8 heads, N = 3072 on a GB300: 4.34 ms with 4 x 4 scalar tiles, 2.80 ms with 8 x 4
+// packed ones (FMA pipe 62% busy, shared wavefronts 63%), 2.40 with 8 x 8 (70%).
+template <int TPT, int NPT>
+struct Tile {
+    static constexpr int TM = 16 * TPT;          // tokens
+    static constexpr int TN = 16 * NPT;          // neurons
+    static constexpr int kBlocks = NPT == 8 ? 1 : 2;   // per SM
+    // floats per k of the activations and of the weights (gate, up): 16-byte rows whose start moves by
+    // half the banks every 4 k, so that the transposing stores do not collide
+    static constexpr int SA = TM + 4;
+    static constexpr int SB = 2 * TN + 4;
+    static constexpr int kStage = TK * (SA + SB);
+    static constexpr int kAb = kThreads * TPT * NPT * 2;   // alpha, beta
+    static constexpr size_t kSmem = sizeof(float) * (2 * kStage + kAb + 8 * TN);
+};
+static_assert(Tile<8, 8>::kSmem <= 227 * 1024 && 2 * (Tile<4, 4>::kSmem + 1024) <= 227 * 1024, "shared memory");
+
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t twice(float v) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
+// Neuron of the thread's j-th column: float4 groups 64 apart.
+__device__ __forceinline__ int col_of(int tx, int j) { return 64 * (j >> 2) + 4 * tx + (j & 3); }
+
+// acc_g[i][p], acc_u[i][p] = sum over k of act[t_i, k] (Wg, Wu)[n_2p, n_2p+1; k] for the thread's tokens
+// t_i = t0 + TPT ty + i and neurons n_j = n0 + col_of(tx, j).  Rows and k beyond the edges read as zero.
+template <int TPT, int NPT>
 __device__ __forceinline__ void tile_gemm(const float* __restrict__ act, int64_t T, int d,
                                           const float* __restrict__ Wg, const float* __restrict__ Wu, int N,
-                                          int64_t t0, int n0, float (&acc_g)[4][4], float (&acc_u)[4][4],
-                                          float (*xs)[TT + 1], float (*gs)[TN + 1], float (*us)[TN + 1]) {
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+                                          int64_t t0, int n0, uint64_t (&acc_g)[TPT][NPT / 2],
+                                          uint64_t (&acc_u)[TPT][NPT / 2], float* stages) {
+    using S = Tile<TPT, NPT>;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    constexpr int kRowsA = TPT / 4, kRowsW = NPT / 4;    // rows per thread
+    const int row = tid >> 2, kq = (tid & 3) * 4;        // 64 rows x 4 float4 per round
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TPT; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc_g[i][j] = 0.0f, acc_u[i][j] = 0.0f;
-    for (int k0 = 0; k0 < d; k0 += TK) {
-        // 64 rows x 16 k per operand: 1024 elements, 4 per thread
+        for (int q = 0; q < NPT / 2; ++q) acc_g[i][q] = acc_u[i][q] = 0;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 ra[kRowsA], rg[kRowsW], ru[kRowsW];
+    const float* pa = act + (t0 + row) * d + kq;
+    const int64_t wo = static_cast<int64_t>(n0 + row) * d + kq;
+    auto fetch = [&](int k0) {
+        const bool k_in = k0 + kq < d;                   // d is a multiple of 8
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int idx = threadIdx.x + e * kThreads;
-            const int r = idx / TK, kk = idx % TK;
-            const int k = k0 + kk;
-            const int64_t t = t0 + r;
-            const int n = n0 + r;
-            xs[kk][r] = (t < T && k < d) ? act[t * d + k] : 0.0f;
-            gs[kk][r] = (n < N && k < d) ? Wg[static_cast<int64_t>(n) * d + k] : 0.0f;
-            us[kk][r] = (n < N && k < d) ? Wu[static_cast<int64_t>(n) * d + k] : 0.0f;
+        for (int e = 0; e < kRowsA; ++e) {
+            const bool in = k_in && t0 + row + 64 * e < T;
+            ra[e] = in ? *reinterpret_cast<const float4*>(pa + 64 * e * static_cast<int64_t>(d) + k0) : zero;
         }
-        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < kRowsW; ++e) {
+            const bool in = k_in && n0 + row + 64 * e < N;
+            const int64_t o = wo + 64 * e * static_cast<int64_t>(d) + k0;
+            rg[e] = in ? *reinterpret_cast<const float4*>(Wg + o) : zero;
+            ru[e] = in ? *reinterpret_cast<const float4*>(Wu + o) : zero;
+        }
+    };
+    auto stash = [&](float* st) {
+        auto put = [](float* to, int stride, const float4& v) {
+            to[0] = v.x, to[stride] = v.y, to[2 * stride] = v.z, to[3 * stride] = v.w;
+        };
+#pragma unroll
+        for (int e = 0; e < kRowsA; ++e) put(st + kq * S::SA + row + 64 * e, S::SA, ra[e]);
+        float* bs = st + TK * S::SA + kq * S::SB + row;
+#pragma unroll
+        for (int e = 0; e < kRowsW; ++e) {
+            put(bs + 64 * e, S::SB, rg[e]);
+            put(bs + S::TN + 64 * e, S::SB, ru[e]);
+        }
+    };
+    fetch(0);
+    stash(stages);
+    __syncthreads();
+    const int blocks = (d + TK - 1) / TK;
+    for (int b = 0; b < blocks; ++b) {
+        const bool more = b + 1 < blocks;
+        if (more) fetch((b + 1) * TK);
+        const float* as = stages + (b & 1) * S::kStage + TPT * ty;
+        const float* bs = stages + (b & 1) * S::kStage + TK * S::SA + 4 * tx;
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
-            float a[4], bg[4], bu[4];
+            uint64_t a[TPT], g[NPT / 2], u[NPT / 2];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = xs[kk][ty + 16 * i];
+            for (int i = 0; i < TPT; i += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(as + kk * S::SA + i);
+                a[i] = twice(v.x), a[i + 1] = twice(v.y), a[i + 2] = twice(v.z), a[i + 3] = twice(v.w);
+            }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) bg[j] = gs[kk][tx + 16 * j], bu[j] = us[kk][tx + 16 * j];
+            for (int q = 0; q < NPT / 4; ++q) {
+                const ulonglong2 vg = *reinterpret_cast<const ulonglong2*>(bs + kk * S::SB + 64 * q);
+                const ulonglong2 vu = *reinterpret_cast<const ulonglong2*>(bs + kk * S::SB + S::TN + 64 * q);
+                g[2 * q] = vg.x, g[2 * q + 1] = vg.y, u[2 * q] = vu.x, u[2 * q + 1] = vu.y;
+            }
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < TPT; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    acc_g[i][j] = fmaf(a[i], bg[j], acc_g[i][j]);
-                    acc_u[i][j] = fmaf(a[i], bu[j], acc_u[i][j]);
+                for (int q = 0; q < NPT / 2; ++q) {
+                    fma2(acc_g[i][q], a[i], g[q]);
+                    fma2(acc_u[i][q], a[i], u[q]);
                 }
         }
+        if (more) stash(stages + ((b + 1) & 1) * S::kStage);   // its last readers passed the previous barrier
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(kThreads)
+// Blocks: `whole` tiles (neuron tile fastest), then the remaining tiles, each split by heads over `split`
+// blocks (each repeats the X pass; the first adds the activation term).
+template <int TPT, int NPT>
+__global__ void __launch_bounds__(kThreads, Tile<TPT, NPT>::kBlocks)
 affinity_fo_f32_kernel(const float* __restrict__ X, const float* __restrict__ C, const float* __restrict__ Wg,
                        const float* __restrict__ Wu, int64_t T, int d, int G, int N, float* __restrict__ partial,
-                       const float* __restrict__ rms, float* __restrict__ partial_act) {
-    __shared__ float xs[TK][TT + 1];
-    __shared__ float gs[TK][TN + 1];
-    __shared__ float us[TK][TN + 1];
-    __shared__ float red[16][TN + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int n0 = blockIdx.x * TN;
-    const int64_t tile = blockIdx.y;
-    const int64_t t0 = tile * TT;
-
-    float acc_g[4][4], acc_u[4][4], alpha[4][4], beta[4][4];
-    tile_gemm(X, T, d, Wg, Wu, N, t0, n0, acc_g, acc_u, xs, gs, us);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float g = acc_g[i][j], u = acc_u[i][j];
-            const float s = 1.0f / (1.0f + expf(-g));
-            beta[i][j] = g * s;
-            alpha[i][j] = s * (1.0f + g * (1.0f - s)) * u;
-        }
-    if (rms) {
-        // down-edge activation term: sum over this tile's tokens of (silu(g) u)^2 / r'^2
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float s = 0.0f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int64_t t = t0 + ty + 16 * i;
-                if (t < T) {
-                    const float act = beta[i][j] * acc_u[i][j];
-                    const float r = rms[t];
-                    s = fmaf(act * act, 1.0f / (r * r), s);
-                }
-            }
-            red[ty][tx + 16 * j] = s;
-        }
-        __syncthreads();
-        if (threadIdx.x < TN) {
-            float s = 0.0f;
-            for (int r = 0; r < 16; ++r) s += red[r][threadIdx.x];
-            const int n = n0 + threadIdx.x;
-            if (n < N) partial_act[tile * N + n] = s;
-        }
-        __syncthreads();
+                       const float* __restrict__ rms, float* __restrict__ partial_act, int64_t whole, int split) {
+    using S = Tile<TPT, NPT>;
+    extern __shared__ __align__(16) float f32_smem[];
+    float* stages = f32_smem;
+    float2* ab = reinterpret_cast<float2*>(f32_smem + 2 * S::kStage);      // [TPT * NPT][threads]
+    float* red = f32_smem + 2 * S::kStage + S::kAb;                        // [8 warps][TN]
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, warp = tid >> 5;
+    int64_t unit = blockIdx.x;
+    int part = 0, parts = 1;
+    if (unit >= whole) {
+        part = static_cast<int>((unit - whole) % split);
+        parts = split;
+        unit = whole + (unit - whole) / split;
     }
-    for (int h = 0; h < G; ++h) {
-        tile_gemm(C + static_cast<int64_t>(h) * T * d, T, d, Wg, Wu, N, t0, n0, acc_g, acc_u, xs, gs, us);
+    const int nt = (N + S::TN - 1) / S::TN;
+    const int n0 = static_cast<int>(unit % nt) * S::TN;
+    const int64_t tile = unit / nt;
+    const int64_t t0 = tile * S::TM;
+    const int h0 = G * part / parts, h1 = G * (part + 1) / parts;
+
+    // sum over the block's tokens of the threads' per-neuron sums, in a fixed order, to dst[n]
+    auto reduce = [&](const float (&s)[NPT], float* dst) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float s = 0.0f;
+        for (int j = 0; j < NPT; ++j) {
+            const float v = s[j] + __shfl_xor_sync(0xFFFFFFFFu, s[j], 16);   // the warp's two token rows
+            if ((tid & 16) == 0) red[warp * S::TN + col_of(tx, j)] = v;
+        }
+        __syncthreads();
+        if (tid < S::TN && n0 + tid < N) {
+            float v = 0.0f;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float dlt = alpha[i][j] * acc_g[i][j] + beta[i][j] * acc_u[i][j];
-                s = fmaf(dlt, dlt, s);
+            for (int w = 0; w < 8; ++w) v += red[w * S::TN + tid];
+            dst[n0 + tid] = v;
+        }
+        // red is rewritten after the next tile_gemm's barriers
+    };
+
+    uint64_t acc_g[TPT][NPT / 2], acc_u[TPT][NPT / 2];
+    tile_gemm<TPT, NPT>(X, T, d, Wg, Wu, N, t0, n0, acc_g, acc_u, stages);
+    {
+        float act[NPT];
+#pragma unroll
+        for (int j = 0; j < NPT; ++j) act[j] = 0.0f;
+        const bool want = rms && part == 0;
+#pragma unroll
+        for (int i = 0; i < TPT; ++i) {
+            const int64_t t = t0 + TPT * ty + i;
+            const float r = want && t < T ? rms[t] : 0.0f;
+            const float ir2 = want && t < T ? 1.0f / (r * r) : 0.0f;
+#pragma unroll
+            for (int j = 0; j < NPT; ++j) {
+                const float2 g2 = unpack2(acc_g[i][j >> 1]), u2 = unpack2(acc_u[i][j >> 1]);
+                const float g = (j & 1) ? g2.y : g2.x, u = (j & 1) ? u2.y : u2.x;
+                const float s = 1.0f / (1.0f + expf(-g));
+                const float beta = g * s;
+                ab[(NPT * i + j) * kThreads + tid] = make_float2(s * (1.0f + g * (1.0f - s)) * u, beta);
+                // down-edge activation term: (silu(g) u)^2 / r'^2
+                if (want && t < T) act[j] = fmaf((beta * u) * (beta * u), ir2, act[j]);
             }
-            red[ty][tx + 16 * j] = s;
         }
-        __syncthreads();
-        if (threadIdx.x < TN) {
-            float s = 0.0f;
-            for (int r = 0; r < 16; ++r) s += red[r][threadIdx.x];
-            const int n = n0 + threadIdx.x;
-            if (n < N) partial[(tile * G + h) * N + n] = s;
-        }
-        __syncthreads();
+        if (want) reduce(act, partial_act + tile * N);
+    }
+    for (int h = h0; h < h1; ++h) {
+        tile_gemm<TPT, NPT>(C + static_cast<int64_t>(h) * T * d, T, d, Wg, Wu, N, t0, n0, acc_g, acc_u, stages);
+        float sum[NPT];
+#pragma unroll
+        for (int j = 0; j < NPT; ++j) sum[j] = 0.0f;
+#pragma unroll
+        for (int i = 0; i < TPT; ++i)
+#pragma unroll
+            for (int j = 0; j < NPT; ++j) {
+                const float2 pg2 = unpack2(acc_g[i][j >> 1]), pu2 = unpack2(acc_u[i][j >> 1]);
+                const float pg = (j & 1) ? pg2.y : pg2.x, pu = (j & 1) ? pu2.y : pu2.x;
+                const float2 w = ab[(NPT * i + j) * kThreads + tid];
+                const float dlt = w.x * pg + w.y * pu;
+                sum[j] = fmaf(dlt, dlt, sum[j]);
+            }
+        reduce(sum, partial + (tile * G + h) * N);
     }
 }
 
@@ -162,25 +256,42 @@ __global__ void f32_reduce_kernel(const float* __restrict__ partial, float* __re
 
 size_t workspace_bytes(int64_t T, int d, int G, int N) {
     (void)d;
-    const int64_t tiles = (T + TT - 1) / TT;
+    const int64_t tiles = (T + kTokMin - 1) / kTokMin;
     return kWorkspaceHeader + static_cast<size_t>(tiles) * (G + 1) * N * sizeof(float);
 }
 
 int launch_grouped(const float* X, const float* C, const float* Wg, const float* Wu, int64_t T, int d, int G, int N,
                    float* A, void* workspace, cudaStream_t stream, const float* rms, float* act2, int qpg) {
     if (qpg < 1 || G % qpg) return DTP_ERR_ARG;
-    const int64_t tiles = (T + TT - 1) / TT;
-    if (tiles > 65535) return DTP_ERR_UNSUPPORTED;
+    const int64_t tiles64 = (T + kTokMin - 1) / kTokMin;
+    if (tiles64 > 65535) return DTP_ERR_UNSUPPORTED;
     float* partial = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace) + kWorkspaceHeader);
-    float* partial_act = partial + tiles * static_cast<int64_t>(G) * N;
+    float* partial_act = partial + tiles64 * static_cast<int64_t>(G) * N;
     const bool want_act = rms && act2;
-    dim3 grid((N + TN - 1) / TN, static_cast<unsigned>(tiles));
-    affinity_fo_f32_kernel<<<grid, kThreads, 0, stream>>>(X, C, Wg, Wu, T, d, G, N, partial,
-                                                          want_act ? rms : nullptr, partial_act);
+    int dev = 0, sms = 0;
+    DTP_CUDA_TRY(cudaGetDevice(&dev));
+    DTP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // 128 x 128 tiles when there are enough for two thirds of the SMs, else 64 x 64 ones; the tiles left
+    // over after the last full round are split by heads so that they spread over the chip
+    const int64_t large_tiles = static_cast<int64_t>((N + 127) / 128) * ((T + 127) / 128);
+    const bool large = 3 * large_tiles >= 2 * sms;
+    const int64_t tiles = large ? (T + 127) / 128 : tiles64;
+    const int64_t units = large ? large_tiles : static_cast<int64_t>((N + 63) / 64) * tiles64;
+    const int64_t slots = large ? sms : 2 * sms;
+    const int64_t whole = units / slots * slots, left = units - whole;
+    int split = 1;
+    if (left > 0) split = static_cast<int>(slots / left < G ? slots / left : G);
+    const int64_t blocks = whole + left * split;
+    if (blocks > 0x7FFFFFFF) return DTP_ERR_UNSUPPORTED;
+    auto kernel = large ? affinity_fo_f32_kernel<8, 8> : affinity_fo_f32_kernel<4, 4>;
+    const size_t smem = large ? Tile<8, 8>::kSmem : Tile<4, 4>::kSmem;
+    DTP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    kernel<<<static_cast<unsigned>(blocks), kThreads, smem, stream>>>(X, C, Wg, Wu, T, d, G, N, partial,
+                                                                     want_act ? rms : nullptr, partial_act, whole, split);
     DTP_CUDA_TRY(cudaGetLastError());
     const int64_t total = static_cast<int64_t>(G / qpg) * N + (want_act ? N : 0);
-    const int blocks = static_cast<int>((total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024);
-    f32_reduce_kernel<<<blocks, 256, 0, stream>>>(partial, A, G, N, tiles, partial_act, want_act ? act2 : nullptr,
+    const int rblocks = static_cast<int>((total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024);
+    f32_reduce_kernel<<<rblocks, 256, 0, stream>>>(partial, A, G, N, tiles, partial_act, want_act ? act2 : nullptr,
                                                   qpg);
     DTP_CUDA_TRY(cudaGetLastError());
     return DTP_OK;

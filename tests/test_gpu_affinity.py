@@ -106,6 +106,22 @@ def test_fp32_parity_ragged(d, G, N, T):
     assert _rel_fro(A, _oracle(L)) <= F32_TOL
 
 
+@pytest.mark.parametrize("d,G,N,T", [
+    (8, 1, 1, 1), (8, 16, 63, 65), (24, 5, 129, 200),     # one k block; heads split over blocks, ragged tiles
+    (16, 3, 2500, 1025), (40, 2, 2561, 1151)])            # 128-token tiles with a remainder on both axes
+def test_fp32_tile_edges_with_down_term(d, G, N, T):
+    """Both tile forms of the fp32 pass and their split by heads, with the activation term; the bound is
+    the fp32 mode's."""
+    L = synth.make_layer(d, G, N, T, seed=d + N, dtype="f32", outliers=False)
+    g = {k: v.to(DEV) for k, v in L.items()}
+    rms = 0.5 + torch.rand(T, generator=torch.Generator().manual_seed(T))
+    A, act2 = dtp.affinity_accumulate_down(g["X"], g["C"], g["W_gate"], g["W_up"], rms.to(DEV))
+    assert _rel_fro(A.cpu().numpy(), _oracle(L)) <= F32_TOL
+    gate, up = L["X"].double() @ L["W_gate"].double().T, L["X"].double() @ L["W_up"].double().T
+    want = ((gate * torch.sigmoid(gate) * up) / rms.double()[:, None]).square().sum(0)
+    assert _rel_fro(act2.cpu().numpy(), want.numpy()) <= F32_TOL
+
+
 def test_zero_tokens_is_a_noop():
     L = synth.make_layer(64, 2, 32, 8, seed=1, dtype="bf16")
     g = {k: v.to(DEV) for k, v in L.items()}
