@@ -99,6 +99,15 @@ def test_bf16_parity_left_over_units_split_by_heads(d, G, N, T):
     assert _rel_fro(A, _oracle(L)) <= BF16_TOL
 
 
+@pytest.mark.parametrize("d,G,N,T", [
+    (128, 8, 3072, 70), (128, 8, 3072, 300),   # fewer units than workers: every unit split by heads
+    (64, 16, 200, 33), (64, 1, 4096, 130),     # more parts than heads, one head
+    (64, 8, 3072, 900)])                       # odd chunk count in the single-CTA form
+def test_bf16_parity_few_units(d, G, N, T):
+    L = synth.make_layer(d, G, N, T, seed=N + T, dtype="bf16", outliers=True)
+    assert _rel_fro(_gpu(L).cpu().numpy(), _oracle(L)) <= BF16_TOL
+
+
 @pytest.mark.parametrize("d,G,N,T", [(328, 3, 300, 333), (64, 2, 65, 70)])
 def test_fp32_parity_ragged(d, G, N, T):
     L = synth.make_layer(d, G, N, T, seed=3, dtype="f32", outliers=True)
