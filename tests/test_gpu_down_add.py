@@ -119,6 +119,16 @@ def test_add_score_weights_beyond_half_of_l2():
     assert _rel(got, ref) <= BF16_TOL and _elementwise_ok(got, ref)
 
 
+@pytest.mark.parametrize("d,N", [(1, 1), (8, 40), (70, 33), (1024, 3072), (1000, 1028), (129, 8)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_down_sqnorm_sizes(d, N, dtype):
+    """Vector and scalar columns, rows that do not fill a block; fp32 sums of d squares: d * 2^-24."""
+    W = torch.randn(d, N, generator=torch.Generator().manual_seed(d + N)).to(dtype)
+    got = dtp.down_sqnorm(W.to(DEV)).cpu().double()
+    want = W.double().square().sum(0)
+    assert torch.all((got - want).abs() <= max(d, 4) * 2.0 ** -24 * want)
+
+
 def test_down_weight_sqnorm_beyond_half_of_l2():
     """gamma' . W_down^T of 128 MiB (d = 4096, N = 16384): single CTAs; two whole column tiles and
     sampled columns (column k of ||b_gk||^2 depends only on column k of W_down)."""
