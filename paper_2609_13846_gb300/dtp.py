@@ -129,8 +129,10 @@ def _check(fn: str, status: int):
 
 
 def _stream(stream=None) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return int(s.cuda_stream)
+    # the raw handle: building a torch.cuda.Stream for it takes 3 us of every call
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return int(stream.cuda_stream)
 
 
 def _keep(t: torch.Tensor, stream) -> torch.Tensor:
@@ -150,7 +152,7 @@ def _device_mask(m, L: int, dev, stream) -> torch.Tensor | None:
 
 
 def _ptr(t: torch.Tensor | None):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -203,10 +205,11 @@ def _check_f32_out(name, t, shape, device):
 def _affinity_shapes(X, C, W_gate, W_up):
     """Check the affinity inputs (contiguous CUDA tensors of one dtype on one device, X [T,d],
     C [H,T,d], W_gate/W_up [N,d]) and return (T, d, H, N)."""
+    index = X.get_device()
     for name, t in (("X", X), ("C", C), ("W_gate", W_gate), ("W_up", W_up)):
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError(f"{name} must be a contiguous CUDA tensor")
-        if t.device != X.device:
+        if t.get_device() != index:
             raise ValueError(f"{name} must be on X's device")
     if not (X.dtype == C.dtype == W_gate.dtype == W_up.dtype):
         raise TypeError("X, C, W_gate and W_up must share one dtype")
