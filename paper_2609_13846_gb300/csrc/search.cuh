@@ -114,6 +114,7 @@ struct Shared {
     int best_idx;
     int64_t red_i64[kWarps];
     int red_int[kWarps];
+    int* beat;                             // where long repairs show that they go on, or null
 };
 
 // The block's dynamic shared memory starts with Shared; the layer's data follow at kData.  Named this
@@ -305,16 +306,6 @@ static __device__ __noinline__ int64_t block_sum_i64(int64_t x) {
     int64_t t = 0;
     for (int i = 0; i < kWarps; ++i) t += sh.red_i64[i];
     return t;
-}
-
-inline __device__ uint32_t block_max_u32(uint32_t x) {
-    Shared& sh = shared();
-    x = __reduce_max_sync(0xFFFFFFFFu, x);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) sh.wsum[0][warp] = x;
-    __syncthreads();
-    return __reduce_max_sync(0xFFFFFFFFu, sh.wsum[0][lane % kWarps]);
 }
 
 // The smallest and the largest of the team's per-thread values (lo and hi), in every thread.
@@ -997,6 +988,7 @@ __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned)
             if (ex == 0) break;
             exchange_graph<DT, SM>(L, tm, -1);
             if (threadIdx.x == 0) {
+                if (sh.beat && (aug & 31) == 31) atomicAdd(sh.beat, 1);
                 unsigned src = 0;
                 for (int l = 0; l < D; ++l)
                     if (sh.count[l] > cap) src |= 1u << l;
@@ -1030,6 +1022,7 @@ __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned)
     for (int round = 0; round < N + 1; ++round) {
         exchange_graph<DT, SM>(L, tm, -1);
         if (threadIdx.x == 0) {
+            if (sh.beat && (round & 31) == 31) atomicAdd(sh.beat, 1);
             for (int a = 0; a < D; ++a)
                 for (int b = 0; b < D; ++b)
                     sh.P[a][b] = (a == b) ? 0 : (sh.w[a][b] ? gain_of(sh.w[a][b]) : kNegInf);
@@ -1628,7 +1621,7 @@ __device__ __forceinline__ void init_shared() {
     for (int i = threadIdx.x; i < 2 * (kBins + kCounters); i += kThreads)
         sh.hist[i / (kBins + kCounters)][i % (kBins + kCounters)] = 0;
     if (threadIdx.x < DMAX) sh.pi[threadIdx.x] = 0;
-    if (threadIdx.x == 0) sh.status = DTP_OK;
+    if (threadIdx.x == 0) sh.status = DTP_OK, sh.beat = nullptr;
 }
 
 // Validity of A [G][N] (from the slice's first neuron), the fixed-point exponent, and the staged scores.
@@ -1976,11 +1969,12 @@ global_pick_kernel(const float* __restrict__ A_all, int G, int N, int64_t n_unl,
 // flag stops later iterations after the first one (after the first) without a
 // strict increase, so the host never waits.
 //
-// One launch per iteration.  A layer's team also sums the columns that its new
+// One launch runs all iterations where every team can be resident (a cooperative launch: the teams wait
+// for each iteration's score; the scores' matrices stay in shared memory), else one iteration each.  A
+// layer's team also sums the columns that its new
 // assignment contributes to its own head step (up edge) and to the next layer's
 // (down edge); whichever of the two teams that feed a head step arrives second
-// (a counter per layer) runs it, and the last head step adds the score.  No
-// block waits for another team.
+// (a counter per layer) runs it, and the last head step adds the score.
 //
 // Ablations (Sec. 3 "Optimiser", Table 4): per-layer flags freeze a layer's
 // heads or neurons at the contiguous start, and `minimize` minimises J.  A
@@ -1999,6 +1993,8 @@ struct ChainState {
     int failed;    // a team of this iteration reported an error
     int heads;     // head steps of this iteration finished
     int64_t prev;
+    int epoch;     // iterations scored, published after everything above and the head partitions
+    int beat;      // counts on while some team is in a long repair
 };
 
 struct ChainArgs {
@@ -2022,6 +2018,7 @@ struct ChainArgs {
     int64_t* J_q;
     double* J;
     int32_t* iters_done;
+    int rounds;             // iterations of this launch; above 1 every team is resident
 };
 
 // Head step of layer i from the sums of layers i and i - 1; the last one of the iteration adds the score.
@@ -2076,6 +2073,7 @@ __device__ void chain_head_step(const ChainArgs& c, int i) {
         part += __ldcg(c.layer_score + j);
         c.arrived[j] = 0;
     }
+    __threadfence();
     const int64_t total = block_sum_i64(part);
     if (tid == 0) {
         ChainState* st = c.st;
@@ -2091,15 +2089,43 @@ __device__ void chain_head_step(const ChainArgs& c, int i) {
             if (total <= st->prev) st->done = 1;
             else st->prev = total;
         }
+        __threadfence();
+        atomicAdd(&st->epoch, 1);
     }
     __syncthreads();
+}
+
+// Thread 0 of a team: waits until iteration `epoch` (counted from this call's start) has been scored.
+// Gives up after kWaitLimitNs without a sign of progress.  True: another iteration follows.
+__device__ __forceinline__ bool wait_scored(const ChainArgs& c, int epoch) {
+    auto load = [](const int* p) {
+        int v;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        return v;
+    };
+    uint64_t t0 = globaltimer_ns();
+    int beat = load(&c.st->beat);
+    while (load(&c.st->epoch) < epoch) {
+        __nanosleep(100);
+        const int now = load(&c.st->beat);
+        if (now != beat) {
+            beat = now;
+            t0 = globaltimer_ns();
+        } else if (globaltimer_ns() - t0 > kWaitLimitNs) {
+            atomicMin(c.ws_status, static_cast<int>(DTP_ERR_NOT_CONVERGED));
+            return false;
+        }
+    }
+    return load(&c.st->done) == 0;
 }
 
 template <int DT, bool SM>
 __global__ void __launch_bounds__(kThreads, 1) chain_iteration_kernel(const ChainArgs c) {
     Shared& sh = shared();
     __shared__ int second[2];
-    // written only after every block of an iteration has read it, so a team's blocks agree
+    __shared__ int go;
+    // between launches done is written only after every block of an iteration has read it, so a team's
+    // blocks agree
     if (*reinterpret_cast<volatile int*>(&c.st->done)) return;
     Team tm = make_team();
     const int i = blockIdx.x / tm.cl;
@@ -2111,19 +2137,12 @@ __global__ void __launch_bounds__(kThreads, 1) chain_iteration_kernel(const Chai
     init_shared();
     const bool has_down = i + 1 < c.Lyr;
     const bool move = !c.move_neurons || c.move_neurons[i];
+    const int rows = has_down ? 2 * G : G;
     team_sync(tm);                     // every block of the team has started: its shared memory may be written
-    if (tid < G) {
-        sh.h[tid] = c.head[i * G + tid];
-        sh.hn[tid] = has_down ? c.head[(i + 1) * G + tid] : -1;
-    }
+    if (tid == 0) sh.beat = &c.st->beat;
     if (tid < DMAX) sh.pi[tid] = c.prices[i * DMAX + tid];
-    __syncthreads();
-    if (tid < 32) list_heads(sh.h, sh.glist, G, G / DT);
-    else if (tid < 64 && has_down) list_heads(sh.hn, sh.gnlist, G, G / DT);
-    __syncthreads();
     L.nU = c.nbuf + i * GN + L.k0;
     L.nD = has_down ? c.nbuf + (c.Lyr + i) * GN + L.k0 : nullptr;
-    const int rows = has_down ? 2 * G : G;
     if (c.vw.rows) {
         uint32_t* qh = staged_hi(L, buf);
         uint16_t* ql = staged_lo(L, buf, c.vw.rows);
@@ -2135,49 +2154,64 @@ __global__ void __launch_bounds__(kThreads, 1) chain_iteration_kernel(const Chai
                 qh[r * L.rnp + k] = static_cast<uint32_t>(v >> kLoBits);
                 ql[r * L.rnp + k] = static_cast<uint16_t>(v & ((1 << kLoBits) - 1));
             }
-        __syncthreads();
         L.qh = qh;
         L.ql = ql;
     }
     const Layer S = gains_of_slice(L, c.vw, tm);
     Team own = make_own(tm);
-    if (move) {
-        build_gain<DT, SM>(S, has_down, c.minimize != 0);
-        team_neuron_step<DT, SM>(L, c.vw, tm, own);
-        if (sh.status == DTP_OK)
-            for (int k = tid; k < L.n; k += kThreads) c.nu[static_cast<int64_t>(i) * N + L.k0 + k] = S.nu[k];
-    } else {                                                // frozen: nu_i stays contiguous
-        for (int k = tid; k < L.n; k += kThreads)
-            S.nu[k] = static_cast<uint8_t>((static_cast<int64_t>(L.k0 + k) * DT) / N);
+    for (int round = 0; round < c.rounds; ++round) {
         __syncthreads();
-    }
-    const bool ok = sh.status == DTP_OK;
-    if (ok) {
-        column_sums<DT, SM>(L, S.nu, tm, rows);
-        team_sum_i64(rows * DT, tm);
-        if (tm.rank == 0 && tid < rows * DT) {
-            const int r = tid / DT, l = tid % DT;
-            int64_t* to = r < G ? c.up_sums : c.down_sums;
-            to[static_cast<int64_t>(i) * GMAX * DMAX + (r < G ? r : r - G) * DT + l] = sh.B[tid];
+        if (tid < G) {
+            sh.h[tid] = __ldcg(c.head + i * G + tid);
+            sh.hn[tid] = has_down ? __ldcg(c.head + (i + 1) * G + tid) : -1;
         }
+        __syncthreads();
+        if (tid < 32) list_heads(sh.h, sh.glist, G, G / DT);
+        else if (tid < 64 && has_down) list_heads(sh.hn, sh.gnlist, G, G / DT);
+        __syncthreads();
+        if (move) {
+            build_gain<DT, SM>(S, has_down, c.minimize != 0);
+            team_neuron_step<DT, SM>(L, c.vw, tm, own);
+            if (sh.status == DTP_OK)
+                for (int k = tid; k < L.n; k += kThreads) c.nu[static_cast<int64_t>(i) * N + L.k0 + k] = S.nu[k];
+        } else {                                            // frozen: nu_i stays contiguous
+            for (int k = tid; k < L.n; k += kThreads)
+                S.nu[k] = static_cast<uint8_t>((static_cast<int64_t>(L.k0 + k) * DT) / N);
+            __syncthreads();
+        }
+        const bool ok = sh.status == DTP_OK;
+        if (ok) {
+            column_sums<DT, SM>(L, S.nu, tm, rows);
+            team_sum_i64(rows * DT, tm);
+            if (tm.rank == 0 && tid < rows * DT) {
+                const int r = tid / DT, l = tid % DT;
+                int64_t* to = r < G ? c.up_sums : c.down_sums;
+                to[static_cast<int64_t>(i) * GMAX * DMAX + (r < G ? r : r - G) * DT + l] = sh.B[tid];
+            }
+        }
+        if (tm.rank == 0) {
+            if (tid == 0 && !ok) {
+                atomicMin(c.ws_status, sh.status);
+                atomicExch(&c.st->failed, 1);
+            }
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) {
+                second[0] = atomicAdd(&c.arrived[i], 1) == (i > 0 ? 1 : 0);
+                second[1] = has_down && atomicAdd(&c.arrived[i + 1], 1) == 1;
+            }
+            __syncthreads();
+            __threadfence();
+            if (second[0]) chain_head_step<DT, SM>(c, i);
+            if (second[1]) chain_head_step<DT, SM>(c, i + 1);
+            if (tid == 0) go = round + 1 < c.rounds && wait_scored(c, round + 1);
+        }
+        team_sync(tm);                 // also: no block goes on while a peer may still read its shared memory
+        const int more = *at_rank(&go, 0);
+        team_sync(tm);
+        if (!more) break;
     }
-    team_sync(tm);                     // no block leaves while a peer may still read its shared memory
-    if (tm.rank != 0) return;
-    if (tid < DMAX) c.prices[i * DMAX + tid] = sh.pi[tid];
-    if (tid == 0 && !ok) {
-        atomicMin(c.ws_status, sh.status);
-        atomicExch(&c.st->failed, 1);
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        second[0] = atomicAdd(&c.arrived[i], 1) == (i > 0 ? 1 : 0);
-        second[1] = has_down && atomicAdd(&c.arrived[i + 1], 1) == 1;
-    }
-    __syncthreads();
-    __threadfence();
-    if (second[0]) chain_head_step<DT, SM>(c, i);
-    if (second[1]) chain_head_step<DT, SM>(c, i + 1);
+    if (tm.rank == 0 && tid < DMAX) c.prices[i * DMAX + tid] = sh.pi[tid];
 }
 
 // The kernels for one device count, on layers in shared memory or (larger than 16 blocks can hold) in

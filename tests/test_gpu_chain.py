@@ -44,11 +44,27 @@ def test_chain_matches_oracle(L, G, N, D, kind):
 
 
 @pytest.mark.parametrize("L,G,N,D,kind", [(2, 8, 4104, 8, "lognormal"), (2, 8, 3864, 8, "integer"),
-                                          (30, 8, 1540, 4, "lognormal")])
+                                          (30, 8, 1540, 4, "lognormal"), (200, 2, 16, 2, "lognormal")])
 def test_chain_layer_splits(L, G, N, D, kind):
-    """Slices of a layer on several blocks (N = 3864 and 4104 at D = 8), and gathered on two of them."""
+    """Slices of a layer on several blocks (N = 3864 and 4104 at D = 8), gathered on two of them, and more
+    layers than can be resident (one launch per iteration)."""
     Su, Sd = _model(L, G, N, seed=L + N, kind=kind)
     _compare(Su, Sd, D, 10)
+
+
+def test_chain_captured_in_a_graph():
+    """The single cooperative launch replays from a CUDA graph with the same result."""
+    Su, Sd = (torch.as_tensor(x, device=DEV).contiguous() for x in _model(5, 8, 768, seed=12))
+    want = dtp.search_chain(Su, Sd, 4, 10)
+    ws = torch.empty(dtp.search_chain_workspace_size(5, 8, 768, 4), dtype=torch.uint8, device=DEV)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = dtp.search_chain(Su, Sd, 4, 10, workspace=ws, check=False)
+    for _ in range(2):
+        g.replay()
+        torch.cuda.synchronize()
+        for k in want:
+            assert torch.equal(got[k], want[k])
 
 
 @pytest.mark.parametrize("iters", [1, 2])
