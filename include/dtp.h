@@ -121,9 +121,9 @@ int dtp_affinity_accumulate_ex(const void* X, const void* C, const void* W_gate,
  *              kernels running concurrently on other streams (for instance the
  *              layout search of the previous layer, which runs on two SMs when the layer's
  *              gains fit in one block's shared memory, else on up to 16).
- *              When the layer's W_gate and W_up fit in half of the L2 cache
- *              the kernel runs as pairs of CTAs, and n is then rounded down
- *              to an even count (at least one pair: 2 CTAs for n = 1)
+ *              The kernel usually runs as pairs of CTAs, and n is then rounded
+ *              down to an even count (when the layer's W_gate and W_up fit in
+ *              half of the L2 cache: at least one pair, 2 CTAs for n = 1)
  *   flags      DTP_AFFINITY_DEFER_REDUCE: launch only the main kernel; its
  *              per-unit partial sums stay in the workspace and
  *              dtp_affinity_reduce adds them into A (and act2) later, possibly

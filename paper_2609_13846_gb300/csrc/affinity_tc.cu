@@ -12,14 +12,12 @@
 //    X or C_h, in each CTA), N = 256 columns (the neuron tile's 128 W_gate
 //    rows in the even CTA, its 128 W_up rows in the odd CTA).  Each SM stages
 //    and reads only half of the weight operand, which keeps the tensor pipe
-//    busier than a single-CTA instruction does.  Used when the weights fit in
-//    L2 with room to spare.
+//    busier than a single-CTA instruction does and moves a third fewer bytes
+//    from L2 per multiply-add.
 //  - single CTAs issuing one tcgen05.mma of cta_group::1 per K step: M = 128
-//    tokens, N = 256 (W_gate and W_up tiles stacked).  Used for layers whose
-//    weights do not fit in L2: there the pairs' placement (a cluster's CTAs
-//    land on neighbouring SMs, consecutive clusters fill one part of the chip
-//    after another) cost the chunk grouping below most of its L2 reuse --
-//    several times the DRAM traffic on a Llama-3.1-8B-shaped layer.
+//    tokens, N = 256 (W_gate and W_up tiles stacked).  Used where the smaller
+//    units leave the busiest SM with less work (short inputs), and where no
+//    cluster of two can be resident.
 // In both, columns [0,128) of a CTA's accumulator are g (or pg) and [128,256)
 // are u (or pu) of the same 128 neurons for that CTA's 128 tokens.
 //
@@ -96,6 +94,7 @@ constexpr uint32_t kTileAct = BT * BK * 2;     // 16 KB activation operand (this
 constexpr uint32_t kTileW = BNEU * BK * 2;     // 16 KB: the W_gate or the W_up rows of a neuron tile
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kBufCols = 256;
+constexpr int64_t kTokensPerLaunch = 4096;   // pairs on weights beyond L2
 constexpr size_t kRedBytes = 2 * 4 * BNEU * sizeof(float);   // [slot][quadrant][neuron]
 
 // Per form: a stage holds kBoxes 64-wide k blocks, each this CTA's activation box and its weight
@@ -727,7 +726,7 @@ static int64_t busiest_passes(int64_t units, int64_t workers, int G) {
     return units / workers * (G + 1) + (G + split - 1) / split + 1;
 }
 
-// Whether a layer whose weights fit in L2 runs as CTA pairs.  A pass takes a pair as long as a single CTA
+// Whether a layer runs as CTA pairs.  A pass takes a pair as long as a single CTA
 // (each SM has the same multiply-adds to do) and is 12% faster in fact: it keeps the tensor pipe 97% busy,
 // a single CTA 87%.  But single CTAs have twice the units of half the tokens to spread over the chip, which
 // wins on short inputs: 777 tokens of a Qwen-shaped layer run 11 single passes against 13 in pairs (69 us
@@ -747,36 +746,28 @@ int launch_grouped(const void* X, const void* C, const void* Wg, const void* Wu,
                    float* A, void* workspace, cudaStream_t stream, const float* rms, float* act2, int qpg,
                    int max_ctas, int defer_reduce) {
     if (qpg < 1 || G % qpg) return DTP_ERR_ARG;
-    CUtensorMap m_wg, m_wu, m_x, m_c;
+    CUtensorMap m_wg, m_wu;
     const cuuint64_t row_stride = static_cast<cuuint64_t>(d) * 2;
     cuuint64_t dw[2] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(N)};
-    cuuint64_t dx[2] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(T)};
-    cuuint64_t dc[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(T), static_cast<cuuint64_t>(G)};
     cuuint64_t s2[1] = {row_stride};
     cuuint64_t s3[2] = {row_stride, row_stride * static_cast<cuuint64_t>(T)};
-    if (!make_map(&m_wg, Wg, 2, dw, s2, BNEU) || !make_map(&m_wu, Wu, 2, dw, s2, BNEU) ||
-        !make_map(&m_x, X, 2, dx, s2, BT) || !make_map(&m_c, C, 3, dc, s3, BT))
-        return DTP_ERR_CUDA;
+    if (!make_map(&m_wg, Wg, 2, dw, s2, BNEU) || !make_map(&m_wu, Wu, 2, dw, s2, BNEU)) return DTP_ERR_CUDA;
 
     Params p;
     p.G = G;
     p.NT = (N + BNEU - 1) / BNEU;
-    p.TC = static_cast<int>((T + BT - 1) / BT);
     p.KB = (d + BK - 1) / BK;
     p.status = reinterpret_cast<int*>(workspace);
-    p.partial = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace) + kWorkspaceHeader);
-    p.T = T;
-    p.rms = (rms && act2) ? rms : nullptr;
-    p.partial_act = p.rms ? reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace) +
-                                                     align_up(workspace_bytes(T, d, G, N), 256))
-                          : nullptr;
+    float* const partial = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace) + kWorkspaceHeader);
+    const bool want_act = rms && act2;
+    float* const partial_act = want_act ? reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace) +
+                                                                   align_up(workspace_bytes(T, d, G, N), 256))
+                                        : nullptr;
 
     int dev = 0, sms = 0, l2 = 0;
     DTP_CUDA_TRY(cudaGetDevice(&dev));
     DTP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     DTP_CUDA_TRY(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
-    // CTA pairs when all weight tiles fit in half of L2 (no chunk grouping needed), single CTAs
-    // otherwise (and wherever no cluster of two can be resident)
     const double tile_bytes = 2.0 * BNEU * d * 2.0;   // W_gate and W_up rows of one neuron tile
     const bool weights_fit = static_cast<double>(p.NT) * tile_bytes <= l2 / 2.0;
     cudaLaunchConfig_t cfg = {};
@@ -790,63 +781,81 @@ int launch_grouped(const void* X, const void* C, const void* Wg, const void* Wu,
     cfg.attrs = attr;
     // CTA pairs resident at once, queried once per device (0: not yet; -1: none can be, for
     // instance on a partition too small for a cluster of two, and the single form runs instead)
-    int resident = 0;
-    if (weights_fit) {
-        static std::atomic<int> resident_cache[64];
-        resident = dev < 64 ? resident_cache[dev].load(std::memory_order_relaxed) : 0;
-        if (resident == 0) {
-            DTP_CUDA_TRY(cudaFuncSetAttribute(affinity_fo_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              static_cast<int>(Form<true>::kSmemBytes)));
-            cfg.gridDim = dim3(static_cast<unsigned>(sms & ~1), 1, 1);
-            cfg.dynamicSmemBytes = Form<true>::kSmemBytes;
-            cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&resident, affinity_fo_tc_kernel<true>, &cfg) != cudaSuccess ||
-                resident < 1) {
-                (void)cudaGetLastError();
-                resident = -1;
-            }
-            if (dev < 64) resident_cache[dev].store(resident, std::memory_order_relaxed);
+    static std::atomic<int> resident_cache[64];
+    int resident = dev < 64 ? resident_cache[dev].load(std::memory_order_relaxed) : 0;
+    if (resident == 0) {
+        DTP_CUDA_TRY(cudaFuncSetAttribute(affinity_fo_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          static_cast<int>(Form<true>::kSmemBytes)));
+        cfg.gridDim = dim3(static_cast<unsigned>(sms & ~1), 1, 1);
+        cfg.dynamicSmemBytes = Form<true>::kSmemBytes;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&resident, affinity_fo_tc_kernel<true>, &cfg) != cudaSuccess || resident < 1) {
+            (void)cudaGetLastError();
+            resident = -1;
         }
+        if (dev < 64) resident_cache[dev].store(resident, std::memory_order_relaxed);
     }
     const int cap = (max_ctas > 0 && max_ctas < sms) ? max_ctas : sms;
-    const bool pair = resident > 0 && prefer_pairs(p.NT, p.TC, G, cap, resident);
+    const bool pair = resident > 0 && (cap >= 2 || weights_fit) &&
+                      prefer_pairs(p.NT, static_cast<int>((T + BT - 1) / BT), G, cap, resident);
     auto kernel = pair ? affinity_fo_tc_kernel<true> : affinity_fo_tc_kernel<false>;
     const size_t smem = pair ? Form<true>::kSmemBytes : Form<false>::kSmemBytes;
     DTP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
     attr[0].val.clusterDim.x = pair ? 2 : 1;
     cfg.dynamicSmemBytes = smem;
     cfg.numAttrs = pair ? 1 : 0;
-    int workers;
     p.KS = pair ? (p.KB + Form<true>::kBoxes - 1) / Form<true>::kBoxes
                 : (p.KB + Form<false>::kBoxes - 1) / Form<false>::kBoxes;
-    if (pair) {
-        p.TU = (p.TC + 1) / 2;
-        // one CTA pair per two SMs (fewer under max_ctas, rounded down to pairs, at least one
-        // pair), and no more pairs than can be resident at once
-        workers = cap / 2 < resident ? cap / 2 : resident;
-        if (workers < 1) workers = 1;
-    } else {
-        p.TU = p.TC;
-        workers = cap;
+    // Pairs on weights beyond L2 take the tokens in launches of about 4096: in one long launch the pairs
+    // drift apart and share fewer of the weight tiles in flight.  d = 4096, N = 14336, 32768 tokens, back to
+    // back at the power cap: single CTAs 40.8 ms, pairs 43.6 in one launch, 38.9 in four, 38.6 in eight;
+    // d = 2560, N = 9728, 16384 tokens: 8.67, 8.10, 8.07, 8.12 (four).
+    const int64_t launches = pair && !weights_fit && T > kTokensPerLaunch
+                                 ? (T + kTokensPerLaunch / 2) / kTokensPerLaunch : 1;
+    const int64_t tokens = launches > 1 ? align_up((T + launches - 1) / launches, 2 * BT) : T;
+    for (int64_t t0 = 0; t0 < T; t0 += tokens) {
+        p.T = T - t0 < tokens ? T - t0 : tokens;
+        p.TC = static_cast<int>((p.T + BT - 1) / BT);
+        const int64_t slot0 = t0 / BT * p.NT;
+        p.partial = partial + slot0 * G * BNEU;
+        p.rms = want_act ? rms + t0 : nullptr;
+        p.partial_act = want_act ? partial_act + slot0 * BNEU : nullptr;
+        CUtensorMap m_x, m_c;
+        cuuint64_t dx[2] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(p.T)};
+        cuuint64_t dc[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(p.T), static_cast<cuuint64_t>(G)};
+        if (!make_map(&m_x, static_cast<const uint8_t*>(X) + t0 * d * 2, 2, dx, s2, BT) ||
+            !make_map(&m_c, static_cast<const uint8_t*>(C) + t0 * d * 2, 3, dc, s3, BT))
+            return DTP_ERR_CUDA;
+        int workers;
+        if (pair) {
+            p.TU = (p.TC + 1) / 2;
+            // one CTA pair per two SMs (fewer under max_ctas, rounded down to pairs, at least one
+            // pair), and no more pairs than can be resident at once
+            workers = cap / 2 < resident ? cap / 2 : resident;
+            if (workers < 1) workers = 1;
+        } else {
+            p.TU = p.TC;
+            workers = cap;
+        }
+        p.units = static_cast<int64_t>(p.NT) * p.TU;
+        // chunk grouping: keep the weight tiles of the units in flight within a third of L2
+        p.cg = 1;
+        if (!weights_fit)
+            while (p.cg < 64 && p.cg < p.TU && (static_cast<double>(workers) / p.cg) * tile_bytes > l2 / 3.0) p.cg *= 2;
+        p.full_rounds = static_cast<int>(p.units / workers);
+        const int left = static_cast<int>(p.units - static_cast<int64_t>(p.full_rounds) * workers);
+        p.split = left > 0 ? (workers / left < G ? workers / left : G) : 1;
+        if (p.split < 1) p.split = 1;
+        p.tail_items = left * p.split;
+        // fewer units than workers: all of them are split by heads (before, they ran whole on as many workers
+        // as units: 64 tokens of a Qwen-shaped layer, 52 us, took the 9 passes of 512 tokens instead of 4)
+        if (p.full_rounds == 0) workers = p.tail_items;
+        cfg.gridDim = dim3(static_cast<unsigned>(pair ? 2 * workers : workers), 1, 1);
+        DTP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, m_wg, m_wu, m_x, m_c, p));
     }
-    p.units = static_cast<int64_t>(p.NT) * p.TU;
-    // chunk grouping: keep the weight tiles of the units in flight within a third of L2
-    p.cg = 1;
-    if (!weights_fit)
-        while (p.cg < 64 && p.cg < p.TU && (static_cast<double>(workers) / p.cg) * tile_bytes > l2 / 3.0) p.cg *= 2;
-    p.full_rounds = static_cast<int>(p.units / workers);
-    const int left = static_cast<int>(p.units - static_cast<int64_t>(p.full_rounds) * workers);
-    p.split = left > 0 ? (workers / left < G ? workers / left : G) : 1;
-    if (p.split < 1) p.split = 1;
-    p.tail_items = left * p.split;
-    // fewer units than workers: all of them are split by heads (before, they ran whole on as many workers
-    // as units: 64 tokens of a Qwen-shaped layer, 52 us, took the 9 passes of 512 tokens instead of 4)
-    if (p.full_rounds == 0) workers = p.tail_items;
-    cfg.gridDim = dim3(static_cast<unsigned>(pair ? 2 * workers : workers), 1, 1);
-    DTP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, m_wg, m_wu, m_x, m_c, p));
     DTP_CUDA_TRY(cudaGetLastError());
     if (defer_reduce) return DTP_OK;
-    return launch_reduce(workspace, T, d, G, N, A, p.rms ? act2 : nullptr, qpg, stream, 0, 0);
+    return launch_reduce(workspace, T, d, G, N, A, want_act ? act2 : nullptr, qpg, stream, 0, 0);
 }
 
 int launch(const void* X, const void* C, const void* Wg, const void* Wu, int64_t T, int d, int G, int N, float* A,

@@ -215,8 +215,8 @@ def test_odd_and_even_token_chunk_counts(T):
 
 @pytest.mark.parametrize("T,max_ctas", [(300, 0), (300, 5), (1000, 151)])
 def test_weights_beyond_half_of_l2(T, max_ctas):
-    """W_gate + W_up of 128 MiB (d = 4096, N = 8192) exceed half of L2, so the kernel runs as
-    single CTAs with chunk grouping; sampled neuron columns against the oracle, and the grid cap
+    """W_gate + W_up of 128 MiB (d = 4096, N = 8192) exceed half of L2, so the kernel groups
+    token chunks; sampled neuron columns against the oracle, and the grid cap
     leaves A bitwise unchanged."""
     d, G, N = 4096, 2, 8192
     L = synth.make_layer(d, G, N, T, seed=60, dtype="bf16")
@@ -229,6 +229,24 @@ def test_weights_beyond_half_of_l2(T, max_ctas):
     ref = _oracle(L, rows=cols)
     got = A[:, torch.as_tensor(cols, device=DEV)].double().cpu().numpy()
     assert _rel_fro(got, ref) <= BF16_TOL
+
+
+@pytest.mark.parametrize("T", [6145, 12500])   # two and three launches, the last ragged; up to 6143 one
+def test_long_input_on_weights_beyond_l2_runs_in_launches(T):
+    """One call on more tokens than a launch takes equals the same tokens streamed in two calls, for both
+    outputs (fp32 sums in another order: a few ulp), and the grid cap changes nothing."""
+    d, G, N = 2048, 2, 8192
+    L = synth.make_layer(d, G, N, T, seed=61, dtype="bf16", device=DEV)
+    rms = 0.5 + torch.rand(T, device=DEV)
+    A, act2 = dtp.affinity_accumulate_down(L["X"], L["C"], L["W_gate"], L["W_up"], rms)
+    B, act2_b = torch.zeros_like(A), torch.zeros_like(act2)
+    for lo, hi in ((0, 5000), (5000, T)):
+        dtp.affinity_accumulate_down(L["X"][lo:hi].contiguous(), L["C"][:, lo:hi].contiguous(), L["W_gate"], L["W_up"],
+                                     rms[lo:hi].contiguous(), A=B, act2=act2_b)
+    assert _rel_fro(A.cpu().numpy(), B.double().cpu().numpy()) <= 2e-6
+    assert _rel_fro(act2.cpu().numpy(), act2_b.double().cpu().numpy()) <= 2e-6
+    capped = dtp.affinity_accumulate(L["X"], L["C"], L["W_gate"], L["W_up"], max_ctas=101)
+    assert torch.equal(capped, A)
 
 
 @pytest.mark.parametrize("max_ctas", [1, 7, 151])
