@@ -34,7 +34,8 @@ __device__ __forceinline__ int64_t unit_mass(uint64_t q, uint64_t total, uint64_
 __global__ void __launch_bounds__(kThreads, 1)
 chain_normalize_kernel(const float* __restrict__ S_up, const float* __restrict__ S_down, int L, int G, int N, int D,
                        int64_t* __restrict__ nbuf, int32_t* __restrict__ head, int32_t* __restrict__ nu,
-                       ChainState* st, int* ws_status, int64_t* J_q, double* J, int32_t* iters_done) {
+                       ChainState* st, int* ws_status, int64_t* J_q, double* J, int32_t* iters_done,
+                       int64_t* __restrict__ tops) {
     Shared& sh = shared();
     Team tm = make_team();
     const int m = blockIdx.x / tm.cl;
@@ -76,11 +77,14 @@ chain_normalize_kernel(const float* __restrict__ S_up, const float* __restrict__
     const uint64_t total = static_cast<uint64_t>(sh.B[0]);
     team_sync(tm);                     // no block leaves while a peer may still read its shared memory
     if (total == 0) {
+        if (threadIdx.x == 0 && tm.rank == 0) tops[m] = 0;
         for (int64_t i = threadIdx.x; i < n; i += kThreads) dst[i] = 0;
         return;
     }
     const int s = __clzll(static_cast<long long>(total));
     const uint64_t mr = static_cast<uint64_t>(~static_cast<unsigned __int128>(0) / (total << s));   // less 2^64
+    if (threadIdx.x == 0 && tm.rank == 0)
+        tops[m] = unit_mass(static_cast<uint64_t>(quantize_bits(amax, e, kNormPreBits)), total, mr, s);
     for_each_a(src, n, [&](int64_t i, float a) {
         dst[i] = unit_mass(static_cast<uint64_t>(quantize_bits(a, e, kNormPreBits)), total, mr, s);
     });
@@ -295,17 +299,17 @@ int launch(const float* A, int layers, int G, int N, int D, int iters, int32_t* 
 
 static int launch_normalize(const float* S_up, const float* S_down, int Lyr, int G, int N, int D, int64_t* nbuf,
                             int32_t* head, int32_t* nu, ChainState* st, int* ws_status, int64_t* J_q, double* J,
-                            int32_t* iters_done, cudaStream_t stream) {
+                            int32_t* iters_done, int64_t* tops, cudaStream_t stream) {
     int dev = 0;
     DTP_CUDA_TRY(cudaGetDevice(&dev));
     Plan p = {};
     p.cl = resident_teams(dev, 4) > 0 ? 4 : 1;
     return launch_teams(chain_normalize_kernel, false, 2 * Lyr - 1, p, stream, S_up, S_down, Lyr, G, N, D, nbuf, head, nu,
-                        st, ws_status, J_q, J, iters_done);
+                        st, ws_status, J_q, J, iters_done, tops);
 }
 
 struct ChainLayout {
-    size_t state, score, prices, arrived, sums, nbuf, gbuf, total;
+    size_t state, score, prices, arrived, sums, tops, nbuf, gbuf, total;
 };
 
 static ChainLayout chain_layout(int Lyr, int G, int N, int D) {
@@ -322,6 +326,8 @@ static ChainLayout chain_layout(int Lyr, int G, int N, int D) {
     x += align_up(static_cast<size_t>(2 * Lyr) * sizeof(int64_t), 256);     // layer scores / edge scores
     o.sums = x;
     x += align_up(static_cast<size_t>(2 * Lyr) * GMAX * DMAX * sizeof(int64_t), 256);
+    o.tops = x;
+    x += align_up(static_cast<size_t>(2 * Lyr) * sizeof(int64_t), 256);
     o.nbuf = x;
     x += align_up(static_cast<size_t>(2 * Lyr - 1) * GN * sizeof(int64_t), 256);
     o.gbuf = x;
@@ -346,6 +352,7 @@ int launch_chain(const float* S_up, const float* S_down, int Lyr, int G, int N, 
     c.G = G;
     c.N = N;
     c.nbuf = reinterpret_cast<int64_t*>(ws + o.nbuf);
+    c.top = reinterpret_cast<int64_t*>(ws + o.tops);
     c.head = head;
     c.nu = nu;
     c.prices = reinterpret_cast<int64_t*>(ws + o.prices);
@@ -367,7 +374,7 @@ int launch_chain(const float* S_up, const float* S_down, int Lyr, int G, int N, 
     // header, state, prices and arrival counters
     DTP_CUDA_TRY(cudaMemsetAsync(ws, 0, o.score, stream));
     rc = launch_normalize(S_up, S_down, Lyr, G, N, D, reinterpret_cast<int64_t*>(ws + o.nbuf), head, nu, c.st,
-                          c.ws_status, J_q, J, iters_done, stream);
+                          c.ws_status, J_q, J, iters_done, reinterpret_cast<int64_t*>(ws + o.tops), stream);
     if (rc != DTP_OK) return rc;
     // all iterations in one launch while every layer's team has its SMs, else one launch each
     int dev = 0;
@@ -396,7 +403,7 @@ int launch_chain_score(const float* S_up, const float* S_down, int Lyr, int G, i
     int64_t* nbuf = reinterpret_cast<int64_t*>(ws + o.nbuf);
     DTP_CUDA_TRY(cudaMemsetAsync(ws, 0, o.prices, stream));
     const int rc = launch_normalize(S_up, S_down, Lyr, G, N, D, nbuf, nullptr, nullptr, st, ws_status, J_q, J, nullptr,
-                                    stream);
+                                    reinterpret_cast<int64_t*>(ws + o.tops), stream);
     if (rc != DTP_OK) return rc;
     chain_edge_kernel<<<2 * Lyr - 1, kThreads, kData, stream>>>(Lyr, G, N, D, nbuf, head, nu, edge, st, ws_status);
     chain_total_kernel<<<1, 32, 0, stream>>>(2 * Lyr - 1, edge, st, J_q, J);

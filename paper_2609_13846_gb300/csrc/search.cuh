@@ -57,8 +57,9 @@ constexpr int kIdxBits = 18;                       // N <= 2^18
 constexpr int64_t kValBias = int64_t(1) << 45;     // |gain| < 2^44 (H_kv <= 16): fits the 46-bit field
 constexpr int64_t kNegInf = INT64_MIN / 4;
 constexpr int kMaxPasses = 24;                      // price passes before the exact repair
-constexpr int kLoBits = 15;                         // a gain is stored as its upper 29 and lower 15 bits
-constexpr int32_t kPriceMax = 1 << 30;              // |price| in units of 2^15
+constexpr int kLoBits = 15;                         // a score row is stored as a value's upper bits and lower 15
+constexpr int kHiBits = 29;                         // a gain as its upper 29 bits (of the layer's largest) and the rest
+constexpr int32_t kPriceMax = 1 << 30;              // |price| in units of 2^sh (Layer::sh)
 constexpr int kBins = 1024;                         // histogram bins (32 groups of 32)
 constexpr int kCounters = 64;                       // counters merged together with a histogram
 constexpr int kPairs = DMAX;                        // first counter of device pairs (28 of them)
@@ -101,8 +102,8 @@ struct Shared {
     int64_t P[DMAX][DMAX];                 // all-pairs max-gain paths
     int64_t bound[DMAX][DMAX];             // a neuron on a with gap <= bound[a][b] for some b is a candidate
     int64_t pi[DMAX];                      // device prices
-    float scale[DMAX];                     // a device's mean gain in units of 2^15 (relative size only)
-    int32_t price[DMAX];                   // prices in units of 2^15, handed from one warp or block to the others
+    float scale[DMAX];                     // a device's mean gain in units of 2^sh (relative size only)
+    int32_t price[DMAX];                   // prices in units of 2^sh, handed from one warp or block to the others
     int count[DMAX];
     int64_t total, J, Jprev;
     int h[GMAX];
@@ -481,7 +482,7 @@ __device__ bool select_threshold(int n, uint32_t lo, uint32_t range, uint32_t ra
 
 // A block's part of a layer.  Scores come as exact integers in two parts, value = hi << 15 | lo: per
 // head in qh, ql (rows [rows][rnp] of the block's slice of neurons, staged once in shared memory when
-// they fit, else null and recomputed from global memory), per device (the gains M) in hi, lo.
+// they fit, else null and recomputed from global memory), per device (the gains M) in hi, lo with gain = hi << sh | lo.
 // Two ways of keeping the gains: `gathered`, block 0 holds those of all neurons and takes the neuron
 // step alone (the others build gains for it and sum columns), or each block holds its slice's and all
 // take the step together.
@@ -490,6 +491,7 @@ struct Layer {
     const int64_t* nU;  // [G][N] from the slice's first neuron (whole-model search)
     const int64_t* nD;  // the same for the down edge, or null
     int G, N, D, cap, e;
+    int sh;             // a gain's low bits (0 .. 15): the upper part has kHiBits at the layer's largest gain
     int n, k0;          // neurons of this block's slice (in a step: of the gains) and the first one's index
     int np;             // column stride of hi and lo
     int rnp;            // row stride of qh and ql
@@ -544,13 +546,13 @@ __device__ __forceinline__ void score_parts(const Layer& L, int r, int k, uint32
 template <bool SM>
 __device__ __forceinline__ int64_t gain_at(const Layer& L, int l, int k) {
     const int i = l * L.np + k;
-    return (static_cast<int64_t>(hi_of<SM>(L)[i]) << kLoBits) | lo_of<SM>(L)[i];
+    return (static_cast<int64_t>(hi_of<SM>(L)[i]) << L.sh) | lo_of<SM>(L)[i];
 }
 
 __device__ __forceinline__ void set_gain(const Layer& L, int l, int k, int64_t m) {
     const int i = l * L.np + k;
-    L.hi[i] = static_cast<int32_t>(m >> kLoBits);
-    L.lo[i] = static_cast<uint16_t>(m & ((1 << kLoBits) - 1));
+    L.hi[i] = static_cast<int32_t>(m >> L.sh);
+    L.lo[i] = static_cast<uint16_t>(m & ((1 << L.sh) - 1));
 }
 
 // Bytes of a slice of np neurons (np a multiple of 16): hi, lo, nu.
@@ -587,8 +589,7 @@ __device__ __noinline__ void build_gain(const Layer& layer, bool down, bool mini
                         hs += h, ls += lo;
                     }
                 }
-                L.hi[l * L.np + k] = static_cast<int32_t>(hs + (ls >> kLoBits));
-                L.lo[l * L.np + k] = static_cast<uint16_t>(ls & ((1u << kLoBits) - 1u));
+                set_gain(L, l, k, (static_cast<int64_t>(hs) << kLoBits) + ls);
             }
         } else {
             int64_t m[DT], r = 0;
@@ -623,9 +624,10 @@ __device__ __noinline__ void neuron_step_d2(const Layer& layer, Team& tm) {
     // bits and a 32-bit key of its low bits and the index (unique); the second is only looked at
     // when the threshold falls between neurons that share the first
     auto diff = [&](int k) -> int64_t { return gain_at<SM>(L, 0, k) - gain_at<SM>(L, 1, k); };
-    auto upper = [](int64_t d) -> uint32_t { return static_cast<uint32_t>(static_cast<int32_t>(d >> 14)) ^ 0x80000000u; };
+    const int cut = L.sh > 1 ? L.sh - 1 : 0;       // |d| < 2^(29 + sh): the upper key has 30 bits and a sign
+    auto upper = [cut](int64_t d) -> uint32_t { return static_cast<uint32_t>(static_cast<int32_t>(d >> cut)) ^ 0x80000000u; };
     auto lower = [&](int64_t d, int k) -> uint32_t {
-        return (static_cast<uint32_t>(d & 0x3FFF) << kIdxBits) |
+        return (static_cast<uint32_t>(d & ((1 << cut) - 1)) << kIdxBits) |
                static_cast<uint32_t>((1 << kIdxBits) - 1 - (L.k0 + k));
     };
     const uint32_t rank = static_cast<uint32_t>(L.cap);
@@ -697,7 +699,7 @@ __device__ __forceinline__ void close_paths(int D) {
     }
 }
 
-// Steps (b) and (c): the assignment at the prices p (units of 2^15) and its repair over the
+// Steps (b) and (c): the assignment at the prices p (units of 2^sh) and its repair over the
 // candidates.  True: L.nu holds the optimal assignment and sh.pi its prices; `unique` then says
 // whether it is certified to be the lexicographically smallest optimum (because every exchange that
 // would put a smaller device earlier loses).  False: L.nu holds the assignment at the prices.
@@ -723,12 +725,12 @@ __device__ __noinline__ bool assign_candidates(const Layer& layer, Team& tm, con
 #pragma unroll
         for (int l = 0; l < DT; ++l) {
             const int i = l * L.np + k;
-            v[l] = (static_cast<int64_t>(hi_of<SM>(L)[i] - p[l]) << kLoBits) + lo_of<SM>(L)[i];
+            v[l] = (static_cast<int64_t>(hi_of<SM>(L)[i] - p[l]) << L.sh) + lo_of<SM>(L)[i];
         }
     };
     if (tid < DT * DT) {
         const int a = tid / DT, b = tid % DT;
-        const float x = tau * fmaxf(sh.scale[a], sh.scale[b]) * static_cast<float>(1 << kLoBits);
+        const float x = tau * fmaxf(sh.scale[a], sh.scale[b]) * static_cast<float>(1 << L.sh);
         sh.bound[a][b] = tau < 0.0f || x >= 1.0e15f ? kBoundMax : static_cast<int64_t>(x);
     }
     __syncthreads();
@@ -890,7 +892,7 @@ __device__ __noinline__ bool assign_candidates(const Layer& layer, Team& tm, con
 #pragma unroll
         for (int l = 0; l < DT; ++l)
             if (l == tid) own = p[l];
-        sh.pi[tid] = (own << kLoBits) + pot;
+        sh.pi[tid] = (own << L.sh) + pot;
     }
     team_counters(tm);
     unique = sh.counters[0] == 0;
@@ -1323,7 +1325,7 @@ __device__ __noinline__ void neuron_step_general(const Layer& L, Team& tm) {
         for (int l = 1; l < DT; ++l) base = sh.pi[l] < base ? sh.pi[l] : base;
 #pragma unroll
         for (int l = 0; l < DT; ++l) {
-            const int64_t x = (sh.pi[l] - base) >> kLoBits;
+            const int64_t x = (sh.pi[l] - base) >> L.sh;
             p[l] = static_cast<int32_t>(x < kPriceMax ? x : kPriceMax);
         }
     }
@@ -1546,6 +1548,7 @@ static __device__ void layer_view(Layer& L, int G, int N, int D, uint8_t* buf, c
     L.D = D;
     L.cap = N / D;
     L.e = 0;
+    L.sh = kLoBits;
     L.np = gains_np(vw, N);
     L.rnp = vw.np;
     L.k0 = static_cast<int>(tm.rank) * vw.np;
@@ -1615,6 +1618,14 @@ __device__ __forceinline__ void team_neuron_step(const Layer& L, const View& vw,
     }
 }
 
+// The low bits of gains of at most `most` (< 2^44).  A fixed 15 leaves a wide layer's normalised masses
+// (2^40 over all entries) some 11 bits above the cut: so many ties at the selection's upper key that
+// most of a step ran on the second key (one layer, N = 14336, D = 8: 10.1 ms fixed, 0.34 ms like this).
+__device__ __forceinline__ int low_bits(int64_t most) {
+    const int bits = 64 - __clzll(most);
+    return bits <= kHiBits ? 0 : (bits - kHiBits < kLoBits ? bits - kHiBits : kLoBits);
+}
+
 // Statuses, prices and both histograms cleared.
 __device__ __forceinline__ void init_shared() {
     Shared& sh = shared();
@@ -1625,7 +1636,7 @@ __device__ __forceinline__ void init_shared() {
 }
 
 // Validity of A [G][N] (from the slice's first neuron), the fixed-point exponent, and the staged scores.
-static __device__ __noinline__ bool layer_prologue(Layer& L, Team& tm, const float* A, uint8_t* buf, const View& vw) {
+__device__ __forceinline__ bool layer_prologue(Layer& L, Team& tm, const float* A, uint8_t* buf, const View& vw) {
     Shared& sh = shared();
     uint32_t* qh = vw.rows ? staged_hi(L, buf) : nullptr;
     uint32_t top = 0;
@@ -1643,6 +1654,7 @@ static __device__ __noinline__ bool layer_prologue(Layer& L, Team& tm, const flo
     int e = 0;
     if (amax > 0.0f) frexpf(amax, &e);
     L.e = e;
+    L.sh = low_bits(static_cast<int64_t>(L.G / L.D) << kFixedBits);
     L.A = A;
     if (qh) {
         uint16_t* ql = staged_lo(L, buf, vw.rows);
@@ -1747,41 +1759,38 @@ __host__ __device__ inline uint64_t fact_u64(int n) {
     return f;
 }
 
-// Completions of a canonical prefix: r heads left, `used` labelled blocks with
-// rem[] places left, D - used blocks not yet opened (cap places each, opened
-// in order): r! / (prod rem! * cap!^(D-used) * (D-used)!).  r <= 16.
-__device__ inline uint64_t rgs_completions(int r, const int* rem, int used, int D, int cap) {
+// Completions of a canonical prefix: r heads left, `used` labelled blocks holding the 8-bit counts cnt,
+// D - used blocks not yet opened (cap places each, opened in order):
+// r! / (prod (cap - cnt)! * cap!^(D-used) * (D-used)!).  r <= 16.
+__device__ inline uint64_t rgs_completions(int r, uint64_t cnt, int used, int D, int cap) {
     uint64_t n = fact_u64(r);
-    for (int l = 0; l < used; ++l) n /= fact_u64(rem[l]);
+    for (int l = 0; l < used; ++l) n /= fact_u64(cap - static_cast<int>((cnt >> (8 * l)) & 255u));
     const int u = D - used;
     const uint64_t fc = fact_u64(cap);
     for (int i = 0; i < u; ++i) n /= fc;
     return n / fact_u64(u);
 }
 
-// The idx-th canonical balanced labelling in lexicographic order (thread-local).
+// The idx-th canonical balanced labelling in lexicographic order.
 __device__ inline bool unrank_canonical(uint64_t idx, int G, int D, int* h) {
     const int cap = G / D;
-    int cnt[DMAX];
-    for (int l = 0; l < DMAX; ++l) cnt[l] = 0;
+    uint64_t cnt = 0;                  // heads placed per block, 8 bits each
     int used = 0;
     for (int k = 0; k < G; ++k) {
         bool placed = false;
         for (int l = 0; l <= used && l < D; ++l) {
-            if (cnt[l] == cap) continue;
-            ++cnt[l];
+            if (static_cast<int>((cnt >> (8 * l)) & 255u) == cap) continue;
+            const uint64_t cnt2 = cnt + (uint64_t(1) << (8 * l));
             const int used2 = l == used ? used + 1 : used;
-            int rem[DMAX];
-            for (int a = 0; a < used2; ++a) rem[a] = cap - cnt[a];
-            const uint64_t c = rgs_completions(G - k - 1, rem, used2, D, cap);
+            const uint64_t c = rgs_completions(G - k - 1, cnt2, used2, D, cap);
             if (idx < c) {
                 h[k] = l;
+                cnt = cnt2;
                 used = used2;
                 placed = true;
                 break;
             }
             idx -= c;
-            --cnt[l];
         }
         if (!placed) return false;
     }
@@ -1819,11 +1828,7 @@ __device__ int64_t team_sum_gains(const Layer& L, const View& vw, bool labels, T
 static __device__ bool set_partition(int64_t pidx, int G, int D) {
     Shared& sh = shared();
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int hh[GMAX];
-        sh.flag = unrank_canonical(static_cast<uint64_t>(pidx), G, D, hh);
-        for (int g = 0; g < G; ++g) sh.h[g] = hh[g];
-    }
+    if (threadIdx.x == 0) sh.flag = unrank_canonical(static_cast<uint64_t>(pidx), G, D, sh.h);
     __syncthreads();
     const bool ok = sh.flag != 0;
     if (ok && threadIdx.x < 32) list_heads(sh.h, sh.glist, G, G / D);
@@ -2000,6 +2005,7 @@ struct ChainState {
 struct ChainArgs {
     int Lyr, G, N;
     const int64_t* nbuf;
+    const int64_t* top;     // [2 Lyr - 1]: each matrix's largest entry
     int32_t* head;
     int32_t* nu;
     int64_t* prices;        // [Lyr][DMAX]
@@ -2138,6 +2144,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_iteration_kernel(const Chai
     const bool has_down = i + 1 < c.Lyr;
     const bool move = !c.move_neurons || c.move_neurons[i];
     const int rows = has_down ? 2 * G : G;
+    // a gain is a sum over one device's heads, minimising over all others'
+    L.sh = low_bits((c.top[i] + (has_down ? c.top[c.Lyr + i] : 0)) * (c.minimize ? G : G / DT));
     team_sync(tm);                     // every block of the team has started: its shared memory may be written
     if (tid == 0) sh.beat = &c.st->beat;
     if (tid < DMAX) sh.pi[tid] = c.prices[i * DMAX + tid];

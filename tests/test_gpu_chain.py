@@ -52,6 +52,15 @@ def test_chain_layer_splits(L, G, N, D, kind):
     _compare(Su, Sd, D, 10)
 
 
+@pytest.mark.parametrize("D", [2, 8])
+@pytest.mark.parametrize("peak", [1.0, 1e3, 1e9])
+def test_chain_gain_split(D, peak):
+    """The gains' low part has 0 to 15 bits by the largest entry; one entry far above the rest takes all bits."""
+    Su, Sd = _model(2, 8, 512, seed=D)
+    Su[0, 3, 17] *= np.float32(peak)
+    _compare(Su, Sd, D, 10)
+
+
 def test_chain_captured_in_a_graph():
     """The single cooperative launch replays from a CUDA graph with the same result."""
     Su, Sd = (torch.as_tensor(x, device=DEV).contiguous() for x in _model(5, 8, 768, seed=12))
