@@ -5,13 +5,14 @@
 //
 //   layout_order_kernel  order[p] = the item at position p when the items are
 //                        listed device by device, each device's in increasing
-//                        index (one block per layer; a counting pass per
-//                        device with a block-wide scan).
+//                        index (one block per layer and list; counts
+//                        scanned over the block).
 //   gather_rows_kernel   dst block b of rows = src block perm[b]  (q/k/v rows,
 //                        gate/up rows)
 //   gather_cols_kernel   dst column block b = src column block perm[b] in
 //                        every row  (o columns; element-wise columns whose
 //                        rows are not a multiple of 16 bytes)
+//   gather_jobs_kernel   both for several matrices in one launch
 //   gather_cols_staged_kernel  the same for element-wise columns (down
 //                        columns, one per neuron) with 16-byte rows of up to
 //                        32 KB: row tiles staged in shared memory, each
@@ -31,25 +32,86 @@ namespace apply {
 
 constexpr int kOrderThreads = 1024;
 
-// One block per layer.  Labels outside [0, D) or a device holding other than
-// n / D items (when `balanced`) set DTP_ERR_ARG in the status word.
+// One list of labels per layer: heads or neurons.
+struct OrderJob {
+    const int32_t* labels;
+    int32_t* order;
+    int n;
+};
+
+// One block per (layer, job).  Labels outside [0, D) or a device holding other than n / D items (when
+// `balanced`) set DTP_ERR_ARG in the status word.
+// Latency-bound.  Up to 8 devices and 65535 items a block scans all devices' counts at once, 16 bits
+// each in two words, so the labels are read twice and one scan replaces D of them; other sizes scan
+// device by device.
 __global__ void __launch_bounds__(kOrderThreads)
-layout_order_kernel(const int32_t* __restrict__ labels, int n, int D, int balanced, int32_t* __restrict__ order,
-                    int* status) {
-    __shared__ int warp_tot[kOrderThreads / 32];
+layout_order_kernel(OrderJob j0, OrderJob j1, int D, int balanced, int* status) {
+    constexpr int kOrderWarps = kOrderThreads / 32;
+    __shared__ uint64_t warp_tot[2][kOrderWarps];
     __shared__ int base;
-    const int32_t* lab = labels + static_cast<int64_t>(blockIdx.x) * n;
-    int32_t* out = order + static_cast<int64_t>(blockIdx.x) * n;
+    const OrderJob j = blockIdx.y == 0 ? j0 : j1;
+    const int n = j.n;
+    const int32_t* lab = j.labels + static_cast<int64_t>(blockIdx.x) * n;
+    int32_t* out = j.order + static_cast<int64_t>(blockIdx.x) * n;
     const int per = (n + kOrderThreads - 1) / kOrderThreads;
-    const int k0 = threadIdx.x * per;
-    const int k1 = min(n, k0 + per);
+    const int k0 = static_cast<int>(min(static_cast<unsigned>(n), threadIdx.x * static_cast<unsigned>(per)));
+    const int k1 = k0 + min(n - k0, per);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool packed = D <= 8 && n <= 65535;
+    uint64_t c[2] = {0, 0};            // packed: devices 0-3 and 4-7
     int bad = 0;
-    for (int k = k0; k < k1; ++k)
-        if (lab[k] < 0 || lab[k] >= D) bad = 1;
+    for (int k = k0; k < k1; ++k) {
+        const int l = lab[k];
+        bad |= l < 0 || l >= D;
+        const uint64_t one = uint64_t(1) << (16 * (l & 3));
+        if (l < 4) c[0] += one;
+        else c[1] += one;
+    }
     bad = __syncthreads_or(bad);
     if (bad) {
         if (threadIdx.x == 0) atomicMin(status, static_cast<int>(DTP_ERR_ARG));
+        return;
+    }
+    if (packed) {
+        uint64_t incl[2] = {c[0], c[1]};
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, incl[i], o);
+                if (lane >= o) incl[i] += y;
+            }
+        if (lane == 31) warp_tot[0][warp] = incl[0], warp_tot[1][warp] = incl[1];
+        __syncthreads();
+        if (warp < 2) {
+            uint64_t w = warp_tot[warp][lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, w, o);
+                if (lane >= o) w += y;
+            }
+            warp_tot[warp][lane] = w;      // inclusive over warps
+        }
+        __syncthreads();
+        int start = 0;
+        uint64_t pos[2] = {0, 0};          // where this thread's next item of each device goes
+#pragma unroll
+        for (int l = 0; l < 8; ++l) {
+            const int total = static_cast<int>((warp_tot[l >> 2][kOrderWarps - 1] >> (16 * (l & 3))) & 0xFFFFu);
+            if (balanced && l < D && total != n / D && threadIdx.x == 0)
+                atomicMin(status, static_cast<int>(DTP_ERR_ARG));
+            pos[l >> 2] += static_cast<uint64_t>(start) << (16 * (l & 3));
+            start += total;
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) pos[i] += (warp > 0 ? warp_tot[i][warp - 1] : 0) + incl[i] - c[i];
+        for (int k = k0; k < k1; ++k) {
+            const int l = lab[k], sft = 16 * (l & 3);
+            const uint64_t p = l < 4 ? pos[0] : pos[1];
+            out[(p >> sft) & 0xFFFFu] = k;
+            if (l < 4) pos[0] += uint64_t(1) << sft;
+            else pos[1] += uint64_t(1) << sft;
+        }
         return;
     }
     if (threadIdx.x == 0) base = 0;
@@ -64,22 +126,22 @@ layout_order_kernel(const int32_t* __restrict__ labels, int n, int D, int balanc
             const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
             if (lane >= o) incl += y;
         }
-        if (lane == 31) warp_tot[warp] = incl;
+        if (lane == 31) warp_tot[0][warp] = static_cast<uint64_t>(incl);
         __syncthreads();
         if (warp == 0) {
-            int w = warp_tot[lane];
+            int w = static_cast<int>(warp_tot[0][lane]);
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int y = __shfl_up_sync(0xFFFFFFFFu, w, o);
                 if (lane >= o) w += y;
             }
-            warp_tot[lane] = w;      // inclusive over warps
+            warp_tot[0][lane] = static_cast<uint64_t>(w);      // inclusive over warps
         }
         __syncthreads();
-        int pos = base + (warp > 0 ? warp_tot[warp - 1] : 0) + incl - cnt;
+        int pos = base + (warp > 0 ? static_cast<int>(warp_tot[0][warp - 1]) : 0) + incl - cnt;
         for (int k = k0; k < k1; ++k)
             if (lab[k] == l) out[pos++] = k;
-        const int total = warp_tot[kOrderThreads / 32 - 1];
+        const int total = static_cast<int>(warp_tot[0][kOrderWarps - 1]);
         __syncthreads();
         if (threadIdx.x == 0) {
             if (balanced && total != n / D) atomicMin(status, static_cast<int>(DTP_ERR_ARG));
@@ -201,6 +263,73 @@ __global__ void gather_cols_kernel(const uint8_t* __restrict__ src, uint8_t* __r
         }
         if (bad) atomicMin(status, static_cast<int>(DTP_ERR_ARG));
     }
+}
+
+// Several matrices of 16-byte rows in one launch: job j's rows follow job j-1's in one list and a warp
+// takes rows of it grid-strided.  block_rows > 0 gathers rows, 0 column blocks of whole 16-byte words.
+constexpr int kMaxJobs = 6;
+
+struct GatherJob {
+    const uint8_t* src;
+    uint8_t* dst;
+    const int32_t* perm;         // [layers][nblocks]
+    uint32_t rows, words;        // per layer; 16-byte words of a row
+    uint32_t block_rows, block_words, nblocks;
+    uint32_t first;              // rows of the jobs before, over all layers
+};
+
+struct GatherJobs {
+    GatherJob job[kMaxJobs];
+    int n;
+    uint32_t total;              // rows of all jobs over all layers
+};
+
+// A lane's words of a row come in batches of kBatch loads, so that they are in flight together.
+template <typename At>
+__device__ __forceinline__ void copy_words(uint4* d, uint32_t words, int lane, At at) {
+    constexpr int kBatch = 4;
+    uint32_t v = lane;
+    for (; v + 32 * (kBatch - 1) < words; v += 32 * kBatch) {
+        uint4 w[kBatch];
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) w[i] = at(v + 32 * i);
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) d[v + 32 * i] = w[i];
+    }
+    for (; v < words; v += 32) d[v] = at(v);
+}
+
+__global__ void __launch_bounds__(256)
+gather_jobs_kernel(const __grid_constant__ GatherJobs g, int* status) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    int bad = 0;
+    for (uint32_t rr = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); rr < g.total; rr += warps) {
+        int ji = 0;
+        while (ji + 1 < g.n && rr >= g.job[ji + 1].first) ++ji;
+        const GatherJob& j = g.job[ji];
+        const uint32_t at = rr - j.first, layer = at / j.rows, row = at - layer * j.rows;
+        const int32_t* pl = j.perm + static_cast<int64_t>(layer) * j.nblocks;
+        uint4* d = reinterpret_cast<uint4*>(j.dst) + static_cast<int64_t>(at) * j.words;
+        if (j.block_rows) {
+            const uint32_t b = row / j.block_rows;
+            const uint32_t pb = static_cast<uint32_t>(__ldg(pl + b));
+            if (pb >= j.nblocks) { bad = 1; continue; }
+            const uint32_t srow = layer * j.rows + pb * j.block_rows + (row - b * j.block_rows);
+            const uint4* s = reinterpret_cast<const uint4*>(j.src) + static_cast<int64_t>(srow) * j.words;
+            copy_words(d, j.words, lane, [&](uint32_t v) { return s[v]; });
+        } else {
+            const uint4* s = reinterpret_cast<const uint4*>(j.src) + static_cast<int64_t>(at) * j.words;
+            const uint32_t bw = j.block_words;
+            for (uint32_t v = lane; v < j.words; v += 32) {
+                const uint32_t b = v / bw;
+                const uint32_t pb = static_cast<uint32_t>(__ldg(pl + b));
+                if (pb >= j.nblocks) { bad = 1; continue; }
+                d[v] = s[pb * bw + (v - b * bw)];
+            }
+        }
+    }
+    if (bad) atomicMin(status, static_cast<int>(DTP_ERR_ARG));
 }
 
 // Element-wise column gather staged through shared memory (rows of a multiple
@@ -359,27 +488,33 @@ gather_cols_staged_kernel(const uint8_t* __restrict__ src, uint8_t* __restrict__
     }
 }
 
-static int grid_for(int64_t work) {
+// 8 warps a block; a warp takes one row, or about 4 KB of rows shorter than 2 KB, and the grid is as
+// large as that makes it (at least what is resident at once).  Blocks that start as others end keep the
+// rows in flight close together in memory: 28 layers of Qwen-shaped weights, rows of 2 and 4 KB, 278 us
+// the whole application against 296 us with 8 resident blocks per SM walking all rows (303 with 4).
+// Rows of 1 KB 63 us against 67, 512 B 75 against 85, 256 B 130 against 149; one row a warp is slower
+// for these (1 KB 75, 512 B 102) and 8 KB a warp slower at 128 B (142 against 126).
+constexpr int64_t kOneRow = 2048, kWarpBytes = 4096;
+
+static int grid_for_rows(int64_t rows, int64_t row_bytes) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
                                                    cudaSuccess)
         return -1;
-    const int64_t want = (work + 255) / 256;
-    const int64_t cap = static_cast<int64_t>(sms) * 8;   // 8 resident 256-thread blocks per SM
-    return static_cast<int>(want < cap ? (want > 0 ? want : 1) : cap);
+    const int64_t most = (rows + 7) / 8;
+    const int64_t resident = static_cast<int64_t>(sms) * 8;   // 8 resident 256-thread blocks per SM
+    int64_t want = row_bytes >= kOneRow ? most : rows * row_bytes / (8 * kWarpBytes);
+    if (want < resident) want = resident;
+    if (want > most) want = most;
+    return static_cast<int>(want < 1 ? 1 : (want < INT32_MAX ? want : INT32_MAX));
 }
 
 int launch_order(const int32_t* labels, int layers, int n, int D, int balanced, int32_t* order, void* workspace,
                  cudaStream_t stream) {
-    layout_order_kernel<<<layers, kOrderThreads, 0, stream>>>(labels, n, D, balanced, order,
-                                                             reinterpret_cast<int*>(workspace));
+    const OrderJob j = {labels, order, n};
+    layout_order_kernel<<<layers, kOrderThreads, 0, stream>>>(j, j, D, balanced, reinterpret_cast<int*>(workspace));
     DTP_CUDA_TRY(cudaGetLastError());
     return DTP_OK;
-}
-
-static int grid_for_rows(int64_t rows) {
-    // 8 warps per block; at most 8 blocks per SM resident
-    return grid_for(rows * 32);
 }
 
 int launch_rows(const void* src, void* dst, int layers, int64_t rows, int64_t row_bytes, int block_rows,
@@ -387,7 +522,7 @@ int launch_rows(const void* src, void* dst, int layers, int64_t rows, int64_t ro
     int* status = reinterpret_cast<int*>(workspace);
     const bool wide = (row_bytes % 16) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0 &&
                       (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
-    const int grid = grid_for_rows(static_cast<int64_t>(layers) * rows);
+    const int grid = grid_for_rows(static_cast<int64_t>(layers) * rows, row_bytes);
     if (grid < 0) return DTP_ERR_CUDA;
     const auto* s = static_cast<const uint8_t*>(src);
     auto* d = static_cast<uint8_t*>(dst);
@@ -488,7 +623,7 @@ int launch_cols(const void* src, void* dst, int layers, int64_t rows, int64_t ro
     int* status = reinterpret_cast<int*>(workspace);
     const auto* s = static_cast<const uint8_t*>(src);
     auto* d = static_cast<uint8_t*>(dst);
-    const int grid = grid_for_rows(static_cast<int64_t>(layers) * rows);
+    const int grid = grid_for_rows(static_cast<int64_t>(layers) * rows, row_bytes);
     if (grid < 0) return DTP_ERR_CUDA;
     const uintptr_t mis = (reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst));
     const bool rows16 = row_bytes % 16 == 0 && (mis & 15) == 0;
@@ -516,6 +651,91 @@ int launch_cols(const void* src, void* dst, int layers, int64_t rows, int64_t ro
                               rows16 && elem_bytes == 1, stream);
     }
     DTP_CUDA_TRY(cudaGetLastError());
+    return DTP_OK;
+}
+
+// Both orders, then all seven matrices: src, dst = q, k, v, o, gate, up, down.
+//
+// Bound by HBM (every byte read and written once) and, per launch, by its ramp and tail.  The matrices
+// whose rows, column blocks and addresses are whole 16-byte words (all but the element-wise down
+// columns, as a rule) go in one launch: 28 Qwen-shaped layers (1.76 GB moved) 296 us against 317 with
+// a launch for each matrix and order (278 with the grid of grid_for_rows).  Matrices that share memory
+// with another's result (a destination that is another's source) keep the launch order, as do more
+// than 2^31 rows.
+int launch_layout(const int32_t* head_part, const int32_t* neuron_dev, int layers, int G, int N, int D,
+                  int q_per_group, int head_dim, int d, int elem_bytes, const void* const* src, void* const* dst,
+                  int32_t* head_order, int32_t* neuron_order, void* workspace, cudaStream_t stream) {
+    int* status = reinterpret_cast<int*>(workspace);
+    const int64_t qrows = static_cast<int64_t>(G) * q_per_group * head_dim;   // q_proj rows, o_proj columns
+    const int64_t kvrows = static_cast<int64_t>(G) * head_dim;
+    const int64_t row = static_cast<int64_t>(d) * elem_bytes;
+    const int qblk = q_per_group * head_dim;
+    const int64_t qblk_bytes = static_cast<int64_t>(qblk) * elem_bytes;
+    const OrderJob heads = {head_part, head_order, G}, neurons = {neuron_dev, neuron_order, N};
+    layout_order_kernel<<<dim3(layers, 2), kOrderThreads, 0, stream>>>(heads, neurons, D, 1, status);
+    DTP_CUDA_TRY(cudaGetLastError());
+
+    // q, k, v rows and o columns by KV group; gate, up rows and down columns by neuron
+    struct Matrix {
+        int64_t rows, row_bytes;
+        int block_rows;             // 0: columns
+        int64_t block_bytes;
+        const int32_t* perm;
+        int nblocks;
+    };
+    const Matrix mats[7] = {{qrows, row, qblk, 0, head_order, G},
+                            {kvrows, row, head_dim, 0, head_order, G},
+                            {kvrows, row, head_dim, 0, head_order, G},
+                            {d, qrows * elem_bytes, 0, qblk_bytes, head_order, G},
+                            {N, row, 1, 0, neuron_order, N},
+                            {N, row, 1, 0, neuron_order, N},
+                            {d, static_cast<int64_t>(N) * elem_bytes, 0, elem_bytes, neuron_order, N}};
+    bool apart = true;
+    int64_t all_rows = 0;
+    for (int i = 0; i < 7; ++i) {
+        const uintptr_t d0 = reinterpret_cast<uintptr_t>(dst[i]);
+        const uintptr_t dn = static_cast<uintptr_t>(layers * mats[i].rows * mats[i].row_bytes);
+        all_rows += layers * mats[i].rows;
+        for (int k = 0; k < 7; ++k) {
+            if (k == i) continue;
+            const uintptr_t s0 = reinterpret_cast<uintptr_t>(src[k]);
+            const uintptr_t e0 = reinterpret_cast<uintptr_t>(dst[k]);
+            const uintptr_t n = static_cast<uintptr_t>(layers * mats[k].rows * mats[k].row_bytes);
+            apart = apart && (d0 + dn <= s0 || s0 + n <= d0) && (d0 + dn <= e0 || e0 + n <= d0);
+        }
+    }
+    GatherJobs g = {};
+    int64_t bytes = 0;
+    bool taken[7] = {};
+    for (int i : {3, 0, 4, 5, 1, 2}) {      // the widest rows first
+        const Matrix& m = mats[i];
+        const uintptr_t bits = reinterpret_cast<uintptr_t>(src[i]) | reinterpret_cast<uintptr_t>(dst[i]) |
+                               static_cast<uintptr_t>(m.row_bytes) | static_cast<uintptr_t>(m.block_bytes);
+        if (!apart || (bits & 15) || all_rows >= (int64_t(1) << 31) || m.row_bytes >= (int64_t(1) << 31)) continue;
+        GatherJob& j = g.job[g.n++];
+        j = {static_cast<const uint8_t*>(src[i]), static_cast<uint8_t*>(dst[i]), m.perm,
+             static_cast<uint32_t>(m.rows), static_cast<uint32_t>(m.row_bytes / 16),
+             static_cast<uint32_t>(m.block_rows), static_cast<uint32_t>(m.block_bytes / 16),
+             static_cast<uint32_t>(m.nblocks), g.total};
+        g.total += static_cast<uint32_t>(layers * m.rows);
+        bytes += layers * m.rows * m.row_bytes;
+        taken[i] = true;
+    }
+    if (g.n > 0) {
+        const int grid = grid_for_rows(g.total, bytes / g.total);
+        if (grid < 0) return DTP_ERR_CUDA;
+            gather_jobs_kernel<<<grid, 256, 0, stream>>>(g, status);
+        DTP_CUDA_TRY(cudaGetLastError());
+    }
+    for (int i = 0; i < 7; ++i) {
+        if (taken[i]) continue;
+        const Matrix& m = mats[i];
+        const int st = m.block_rows ? launch_rows(src[i], dst[i], layers, m.rows, m.row_bytes, m.block_rows, m.perm,
+                                                  m.nblocks, workspace, stream)
+                                    : launch_cols(src[i], dst[i], layers, m.rows, m.row_bytes, m.block_bytes,
+                                                  elem_bytes, m.perm, m.nblocks, workspace, stream);
+        if (st != DTP_OK) return st;
+    }
     return DTP_OK;
 }
 

@@ -5,6 +5,8 @@ rounded once to bf16: relative Frobenius error <= 5e-3 against the fp64 oracle
 on the same bf16 inputs.  Layout application: index work, so the order and the
 permuted weights are bit-exact against the oracle's.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -120,6 +122,53 @@ def test_apply_layout_bit_exact(d, Hq, G, hd, N, D):
     np.testing.assert_array_equal(no.cpu().numpy(), rno)
     for k in ("q", "k", "v", "o", "gate", "up", "down"):
         assert torch.equal(out[k].cpu().float(), torch.as_tensor(ref[k], dtype=torch.float32)), k
+
+
+@pytest.mark.parametrize("layers,n,D", [(2, 1025, 5), (1, 65528, 8), (1, 65544, 8), (2, 99, 9), (1, 7, 1)])
+def test_layout_order_scan_forms(layers, n, D):
+    """All devices' counts in one packed scan (D <= 8, n <= 65535) and device by device beyond."""
+    test_layout_order_bit_exact(layers, n, D)
+
+
+# rows and columns of whole 16-byte words share a launch: all of them; none (d = 9); the rows alone
+# (4-byte o blocks); the o columns alone (d = 20, 40-byte rows); a row of more than one batch and a tail
+@pytest.mark.parametrize("Lyr,d,q,G,hd,N,D", [(3, 8, 2, 4, 4, 12, 2), (2, 9, 1, 4, 8, 12, 4), (1, 1112, 1, 3, 2, 21, 3),
+                                              (2, 20, 2, 2, 8, 10, 2), (1, 2088, 3, 8, 8, 1000, 8)])
+@pytest.mark.parametrize("chained", [False, True])
+def test_apply_layout_shared_launch(Lyr, d, q, G, hd, N, D, chained):
+    """The gathers by index; `chained`: v is written over the source of k, up over the source of gate."""
+    shapes = dict(q=(G * q * hd, d), k=(G * hd, d), v=(G * hd, d), o=(d, G * q * hd), gate=(N, d), up=(N, d), down=(d, N))
+    gen = torch.Generator().manual_seed(d)
+    W = {k: torch.randn((Lyr, *s), generator=gen).to(torch.bfloat16).to(DEV) for k, s in shapes.items()}
+    h, nu = (torch.as_tensor(x, device=DEV) for x in ablation.random_layout(Lyr, G, N, D, d))
+    ho = torch.argsort(h, dim=1, stable=True)
+    no = torch.argsort(nu, dim=1, stable=True)
+
+    def blocks(x, order, n, dim):        # x's n equal blocks along dim in the given order
+        y = x.unflatten(dim, (n, -1))
+        return torch.stack([y[i].index_select(dim - 1, order[i]) for i in range(Lyr)]).flatten(dim, dim + 1)
+
+    want = {k: blocks(W[k], ho, G, 1) for k in "qkv"}
+    want |= {"o": blocks(W["o"], ho, G, 2), "gate": blocks(W["gate"], no, N, 1), "up": blocks(W["up"], no, N, 1),
+             "down": blocks(W["down"], no, N, 2)}
+    if not chained:
+        out, oh, on = dtp.apply_layout(W, h, nu, D, hd)
+    else:
+        names = list(shapes)
+        out = {k: torch.empty_like(W[k]) for k in names}
+        out["v"] = W["k"]
+        out["up"] = W["gate"]
+        oh, on = torch.empty_like(h), torch.empty_like(nu)
+        ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+        vp7 = ctypes.c_void_p * 7
+        st = dtp.lib().dtp_apply_layout(h.data_ptr(), nu.data_ptr(), Lyr, G, N, D, q, hd, d, 2,
+                                        vp7(*[W[k].data_ptr() for k in names]), vp7(*[out[k].data_ptr() for k in names]),
+                                        oh.data_ptr(), on.data_ptr(), ws.data_ptr(), ws.numel(),
+                                        torch.cuda.current_stream().cuda_stream)
+        assert st == 0 and dtp.workspace_status(ws) == 0
+    assert torch.equal(oh.long(), ho) and torch.equal(on.long(), no)
+    for k in shapes:
+        assert torch.equal(out[k], want[k]), k
 
 
 def test_apply_layout_batched_over_layers_and_dense_function():
