@@ -41,7 +41,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-
 #include "dtp_common.cuh"
 
 namespace dtp {
@@ -69,8 +68,8 @@ constexpr int64_t kBoundMax = int64_t(1) << 50;     // above any difference of r
 constexpr int kStates = 1024;                       // head-step states (G/D + 1)^D of every accepted size
 constexpr int kMaxCluster = 16;
 constexpr int kSums = 2 * GMAX * DMAX + 8;           // int64 sums of one exchange
-// Dynamic shared memory of a block: the slice of M, nu and (if it fits) A.  The static part
-// (struct Shared) takes up to 43 KB of the 227 KB.
+// A block's slice of the gains, nu and (if they fit) the scores; struct Shared before it takes up to
+// 43 KB of the 227 KB.
 constexpr size_t kSmemBudget = 184 * 1024;
 // Layers of up to this many bytes of int64 gains and int32 labels need no global buffer even
 // without clusters (the workspace's size rule; the kernels' own layout is smaller).
