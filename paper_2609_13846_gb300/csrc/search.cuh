@@ -1427,7 +1427,7 @@ __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, 
     const int pairs = rows * DT;                                // at most 256
     int tpp = 32;
     while (tpp * pairs > kThreads) tpp >>= 1;
-    for (int i = tid; i < pairs * tpp; i += kThreads) {         // whole warps: pairs * tpp % 32 == 0 or one round
+    for (int i = tid; i < pairs * tpp; i += kThreads) {         // whole groups of tpp lanes
         const int pair = i / tpp, sub = i % tpp;
         const int r = pair / DT, l = pair % DT;
         const int len = sh.clen[l];
@@ -1440,9 +1440,10 @@ __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, 
             hs += h;
             ls += lo;
         }
+        // the group's own lanes: their lists differ in length, so they need not leave the loop together
+        const unsigned group = (0xFFFFFFFFu >> (32 - tpp)) << (lane & ~(tpp - 1));
         int64_t v = (hs << kLoBits) + ls;
-        const unsigned mask = __activemask();
-        for (int o = tpp >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+        for (int o = tpp >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(group, v, o);
         if (sub == 0) sh.xl[tm.lph][pair] = v;
     }
 }

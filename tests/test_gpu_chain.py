@@ -52,6 +52,15 @@ def test_chain_layer_splits(L, G, N, D, kind):
     _compare(Su, Sd, D, 10)
 
 
+@pytest.mark.parametrize("L,G,N,D", [(3, 16, 20, 4), (2, 16, 34, 2), (2, 12, 60, 4), (2, 12, 66, 6), (2, 8, 1544, 8),
+                                     (2, 16, 1540, 4)])
+def test_chain_column_sum_groups(L, G, N, D):
+    """Groups of 2 to 32 lanes add a (row, device) list each, several in a warp, with lists whose length is
+    no multiple of the group's and (slices of a layer on several blocks) differs from device to device."""
+    Su, Sd = _model(L, G, N, seed=G + N + D)
+    _compare(Su, Sd, D, 10)
+
+
 @pytest.mark.parametrize("D", [2, 8])
 @pytest.mark.parametrize("peak", [1.0, 1e3, 1e9])
 def test_chain_gain_split(D, peak):
