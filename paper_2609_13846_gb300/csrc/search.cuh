@@ -2033,7 +2033,8 @@ __device__ void chain_head_step(const ChainArgs& c, int i) {
     Shared& sh = shared();
     const int G = c.G, tid = threadIdx.x;
     __shared__ int last;
-    const bool failed = *reinterpret_cast<volatile int*>(&c.st->failed) != 0;
+    // another team may set the flag at any time: one thread reads it, and the whole block takes one side
+    const bool failed = __syncthreads_or(tid == 0 && *reinterpret_cast<volatile int*>(&c.st->failed) != 0);
     if (!failed) {
         if (tid < G * DT) {
             int64_t b = __ldcg(c.up_sums + static_cast<int64_t>(i) * GMAX * DMAX + tid);

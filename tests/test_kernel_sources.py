@@ -17,3 +17,19 @@ def test_warp_collectives_name_their_lanes():
     """No collective takes the lanes that happen to be converged for the lanes that take part."""
     for path in glob.glob(os.path.join(CSRC, "*.cu*")):
         assert "__activemask" not in _source(os.path.basename(path)), path
+
+
+def test_flag_of_other_teams_is_read_by_one_thread():
+    """ChainState::failed changes while blocks run: threads that read it for themselves could part at a barrier."""
+    text = _source("search.cuh")
+    reads = [m.start() for m in re.finditer(r"volatile int\*>\(&[\w.>-]*failed\)", text)]
+    assert len(reads) == 2
+    for pos in reads:
+        start = max(text.rfind(c, 0, pos) for c in ";{}")
+        block, depth = [], 0
+        for i in range(pos, -1, -1):          # heads of the blocks around the statement
+            depth += (text[i] == "}") - (text[i] == "{")
+            if depth < 0:
+                depth = 0
+                block.append(text[max(text.rfind(c, 0, i) for c in ";{}") + 1:i])
+        assert "tid == 0" in text[start:pos] or any("tid == 0" in b for b in block)
