@@ -1877,7 +1877,7 @@ global_items_kernel(const float* __restrict__ A_all, int layers, int G, int N, i
                 values[item] = -1;
                 atomicMin(ws_status, sh.status);
             }
-            __syncthreads();
+            team_sync(tm);             // the peers have read block 0's status: the next item resets it
             continue;
         }
         const int64_t v = team_sum_gains<DT, SM>(L, vw, true, tm, own);

@@ -33,3 +33,15 @@ def test_flag_of_other_teams_is_read_by_one_thread():
                 depth = 0
                 block.append(text[max(text.rfind(c, 0, i) for c in ";{}") + 1:i])
         assert "tid == 0" in text[start:pos] or any("tid == 0" in b for b in block)
+
+
+def test_failed_item_ends_at_a_team_barrier():
+    """The exact optimum's blocks copy block 0's status after a step; block 0 resets it for the next item, so no
+    way out of an item after the step may skip the barrier of the team."""
+    text = _source("search.cuh")
+    body = text[text.index("global_items_kernel(const float*"):]
+    body = body[body.index("team_neuron_step<DT, SM>"):body.index("template <")]
+    assert body.count("continue;") == 1
+    for part in body.split("continue;")[:-1]:
+        assert "team_sync(tm)" in part[part.rindex("if (sh.status != DTP_OK)"):]
+    assert "team_sync(tm)" in body.split("continue;")[-1]
