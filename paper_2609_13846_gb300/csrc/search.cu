@@ -220,6 +220,7 @@ static int make_plan(int64_t teams, int rows, int N, int D, Plan* p) {
     int cl = 1;
     while (cl < kMaxCluster && slice_bytes(slice_np(N, cl), D) > kSmemBudget) cl *= 2;
     if (cl > most || slice_bytes(slice_np(N, cl), D) > kSmemBudget) {
+        if (fits_block(N, D)) return DTP_ERR_WORKSPACE;   // no room was asked for: never with the budgets above
         p->cl = 1;
         p->global = 1;
         p->dyn = 0;

@@ -74,6 +74,9 @@ constexpr size_t kSmemBudget = 184 * 1024;
 // Layers of up to this many bytes of int64 gains and int32 labels need no global buffer even
 // without clusters (the workspace's size rule; the kernels' own layout is smaller).
 constexpr size_t kWorkspaceFree = 220 * 1024;
+// One block holds every such layer: its np <= N + 15 neurons of 6 D + 1 bytes (slice_bytes) take less than
+// 3/4 of N's 8 D + 4 and 15 neurons more.  So a layer that lives in the workspace has room there.
+static_assert(kWorkspaceFree / 4 * 3 + 15 * (6 * DMAX + 1) <= kSmemBudget, "layers without a workspace fit one block");
 
 struct Shared {
     uint32_t hist[2][kBins + kCounters];   // this block's counts, two phases

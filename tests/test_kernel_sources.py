@@ -3,6 +3,11 @@ only when warps happen to be scheduled badly, so the sources themselves are read
 import glob
 import os
 import re
+import subprocess
+
+import pytest
+
+from paper_2609_13846_gb300 import build
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_13846_gb300", "csrc")
 
@@ -45,3 +50,18 @@ def test_failed_item_ends_at_a_team_barrier():
     for part in body.split("continue;")[:-1]:
         assert "team_sync(tm)" in part[part.rindex("if (sh.status != DTP_OK)"):]
     assert "team_sync(tm)" in body.split("continue;")[-1]
+
+
+@pytest.mark.parametrize("budget,builds", [(184, True), (166, True), (160, False), (4, False)])
+def test_shared_memory_budget_and_workspace_rule_agree(tmp_path, budget, builds):
+    """Layers that ask for no workspace must fit one block: a budget too small for that does not build."""
+    text = open(os.path.join(CSRC, "search.cuh")).read()
+    line = "constexpr size_t kSmemBudget = 184 * 1024;"
+    assert text.count(line) == 1
+    (tmp_path / "search.cuh").write_text(text.replace(line, f"constexpr size_t kSmemBudget = {budget} * 1024;"))
+    (tmp_path / "t.cu").write_text('#include "search.cuh"\n')
+    cmd = [build.nvcc(), *build.ARCH, "-std=c++17", "-I", os.path.join(build.ROOT, "include"), "-I", CSRC, "-c",
+           str(tmp_path / "t.cu"), "-o", str(tmp_path / "t.o")]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert (r.returncode == 0) == builds, r.stderr
+    assert builds or "layers without a workspace fit one block" in r.stderr
