@@ -10,6 +10,7 @@ import torch
 
 import oracle
 from paper_2609_13846_gb300 import dtp, synth
+from test_gpu_search import WIDEST, only_optimum
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -83,6 +84,30 @@ def test_chain_captured_in_a_graph():
         torch.cuda.synchronize()
         for k in want:
             assert torch.equal(got[k], want[k])
+
+
+@pytest.mark.parametrize("G,N,D", WIDEST)
+def test_chain_widest_layers(G, N, D):
+    """One iteration on three layers: certified neuron steps, the oracle's head steps and score on them."""
+    Su, Sd = _model(3, G, N, seed=N)
+    up, down = [oracle.normalize_unit_mass(S) for S in Su], [oracle.normalize_unit_mass(S) for S in Sd]
+    h0 = np.arange(G) * D // G
+    r = dtp.search_chain(torch.as_tensor(Su, device=DEV), torch.as_tensor(Sd, device=DEV), D, 1)
+    h, nu = r["h"].cpu().numpy(), r["nu"].cpu().numpy()
+    for i in range(3):
+        gain = up[i] + down[i] if i < 2 else up[i]
+        assert only_optimum(np.stack([gain[h0 == l].sum(axis=0) for l in range(D)], axis=1), nu[i])
+        fed = [(up[i], nu[i])] + ([(down[i - 1], nu[i - 1])] if i > 0 else [])
+        want, _ = oracle.head_step(np.concatenate([f[0] for f in fed], axis=1), np.concatenate([f[1] for f in fed]), D)
+        np.testing.assert_array_equal(h[i], want)
+    assert int(r["J_q"]) == oracle.chain_score(Su, Sd, h, nu)
+
+
+@pytest.mark.parametrize("N", [131072, 231700])
+def test_chain_widest_layers_converge(N):
+    """All iterations in one launch on two devices: 16 blocks a layer, and gains in global memory."""
+    Su, Sd = _model(2, 2, N, seed=N)
+    _compare(Su, Sd, 2, 10)
 
 
 @pytest.mark.parametrize("iters", [1, 2])

@@ -84,15 +84,55 @@ def test_full_size_qwen_d2_and_d4():
 @pytest.mark.parametrize("G,N,D,kind", [
     (8, 776, 4, "lognormal"), (8, 1544, 4, "lognormal"), (6, 9000, 3, "integer"),   # one block and two, a gathered layer
     (8, 4096, 8, "integer"), (8, 4096, 8, "lognormal"), (4, 16400, 4, "lognormal"),  # slices on several blocks
-    (2, 262144, 2, "lognormal")])                                                    # gains in global memory
+    (2, 131072, 2, "lognormal"), (2, 131072, 2, "integer"),                          # clusters of 16 blocks
+    (2, 262144, 2, "lognormal"), (4, 231700, 2, "integer")])                         # gains in global memory
 def test_search_layer_splits(G, N, D, kind):
     """How a layer is spread over blocks: sizes on both sides of each line, with and without ties."""
     A = synth.make_affinity_matrix(G, N, seed=G + N + D, kind=kind).numpy()
     _compare(A, D, 10)
 
 
+def only_optimum(M, nu):
+    """nu is balanced and the only maximiser of sum_k M[k, nu(k)]: every cycle of exchanges between devices
+    loses.  N D steps where the oracle's successive paths take N^2 D, for layers too wide for it."""
+    N, D = M.shape
+    assert (np.bincount(nu, minlength=D) == N // D).all()
+    w = np.full((D, D), -(1 << 60), dtype=np.int64)
+    for a in range(D):
+        w[a] = (M[nu == a] - M[nu == a][:, a:a + 1]).max(axis=0)
+        w[a, a] = -(1 << 60)
+    for c in range(D):
+        w = np.maximum(w, w[:, c:c + 1] + w[c:c + 1, :])
+    return bool((np.diagonal(w) < 0).all())
+
+
+# 16 blocks, then gains in global memory: with 16-bit lists of neurons, and with 32-bit ones
+WIDEST = [(8, 40000, 8), (8, 61448, 8), (8, 65544, 8), (4, 120580, 4)]
+
+
+@pytest.mark.parametrize("G,N,D", WIDEST)
+def test_widest_layers(G, N, D):
+    """One iteration: the neuron step from the contiguous heads, certified, and the oracle's head step on it."""
+    A = synth.make_affinity_matrix(G, N, seed=N).numpy()
+    q, _ = oracle.quantize(A)
+    h0 = np.arange(G) * D // G
+    M = np.stack([q[h0 == l].sum(axis=0) for l in range(D)], axis=1)
+    r = dtp.search_layout(torch.as_tensor(A, device=DEV), D, 1)
+    nu = r["nu"].cpu().numpy()
+    assert only_optimum(M, nu)
+    h, score = oracle.head_step(q, nu, D)
+    np.testing.assert_array_equal(r["h"].cpu().numpy(), h)
+    assert int(r["score_q"]) == score
+    # of these layers' exact optimum only G == D is quick on the host: one unlabelled partition
+    if G == D:
+        g = dtp.search_global(torch.as_tensor(A, device=DEV), D)
+        np.testing.assert_array_equal(g["h"].cpu().numpy(), h0)
+        np.testing.assert_array_equal(g["nu"].cpu().numpy(), nu)
+        assert int(g["score_q"]) == oracle.layout_score(q, h0, nu)
+
+
 def test_full_size_llama_neuron_count_d8():
-    """Llama-3.1-8B shape N=14336 (global-memory path of the search), D=8."""
+    """Llama-3.1-8B shape N=14336 (slices of the layer on the blocks of a cluster), D=8."""
     A = synth.make_affinity_matrix(8, 14336, seed=3).numpy()
     _compare(A, 8, 10, unique=True)
 
@@ -134,13 +174,24 @@ def test_global_layout_matches_oracle(G, N, D, layers, kind):
 
 
 def test_global_layout_llama_width():
-    """N = 14336 (Llama-3.1-8B): M and nu do not fit in shared memory; per-block global buffers."""
+    """N = 14336 (Llama-3.1-8B): a layer does not fit one block's shared memory; slices on several blocks."""
     A = synth.make_affinity_matrix(8, 14336, seed=3).numpy()
     r = dtp.search_global(torch.as_tensor(A, device=DEV), 4)
     ref = oracle.global_layout(A, 4)
     np.testing.assert_array_equal(r["h"].cpu().numpy(), ref["h"])
     np.testing.assert_array_equal(r["nu"].cpu().numpy(), ref["nu"])
     assert int(r["score_q"]) == ref["score_q"]
+
+
+def test_global_layout_of_layers_in_global_memory():
+    """Two layers of three partitions each, every item on its own buffer in the workspace."""
+    As = np.stack([synth.make_affinity_matrix(4, 231700, seed=i).numpy() for i in range(2)])
+    r = dtp.search_global(torch.as_tensor(As, device=DEV), 2)
+    for i in range(2):
+        ref = oracle.global_layout(As[i], 2)
+        np.testing.assert_array_equal(r["h"][i].cpu().numpy(), ref["h"])
+        np.testing.assert_array_equal(r["nu"][i].cpu().numpy(), ref["nu"])
+        assert int(r["score_q"][i]) == ref["score_q"]
 
 
 def test_global_layout_rejects_invalid_entries():
