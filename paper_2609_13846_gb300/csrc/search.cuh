@@ -101,6 +101,7 @@ struct Shared {
     uint64_t E[DMAX][DMAX];                // candidate exchange graph: packed (gain, slot), 0 = none
     uint64_t wl[2][DMAX * DMAX];           // exchange graph over all neurons of the slice, two phases
     uint64_t w[DMAX][DMAX];                // the team's (0 = no neuron on the source device)
+    uint64_t wk[DMAX][DMAX];               // and over the neurons above an index
     int64_t P[DMAX][DMAX];                 // all-pairs max-gain paths
     int64_t bound[DMAX][DMAX];             // a neuron on a with gap <= bound[a][b] for some b is a candidate
     int64_t pi[DMAX];                      // device prices
@@ -113,7 +114,7 @@ struct Shared {
     int glist[GMAX], gnlist[GMAX];         // heads listed device by device, for h and for hn
     int status;
     int flag;
-    unsigned dirty;
+    unsigned dirty;                        // devices whose edges of E or w are to be found again
     int best_idx;
     int64_t red_i64[kWarps];
     int red_int[kWarps];
@@ -901,20 +902,24 @@ __device__ __noinline__ bool assign_candidates(const Layer& layer, Team& tm, con
     return true;
 }
 
-// Exchange graph over the team's neurons with index > lo: sh.w[a][b] = packed
-// (max gain of moving such a neuron from a to b, lowest index among ties).
+// Exchange graph over the team's neurons with index > lo: w[a][b] = packed (max gain of moving such a
+// neuron from a to b, lowest index among ties).  lo < 0: all neurons, into sh.w, only the edges out of the
+// devices in sh.dirty (the others stand from before); else into sh.wk.
 template <int DT, bool SM>
 __device__ __noinline__ void exchange_graph(const Layer& L, Team& tm, int lo) {
     Shared& sh = shared();
     uint64_t* wl = sh.wl[tm.wph];
+    const unsigned rows = lo < 0 ? sh.dirty : (1u << DT) - 1u;
+    const int first = lo < L.k0 ? 0 : lo + 1 - L.k0;
     if (threadIdx.x < DMAX * DMAX) wl[threadIdx.x] = 0;
     __syncthreads();
     for (int a = 0; a < DT; ++a) {
+        if (!((rows >> a) & 1u)) continue;
         uint64_t best[DT];
 #pragma unroll
         for (int b = 0; b < DT; ++b) best[b] = 0;
-        for (int k = threadIdx.x; k < L.n; k += kThreads) {
-            if (L.k0 + k <= lo || nu_of<SM>(L)[k] != a) continue;
+        for (int k = first + threadIdx.x; k < L.n; k += kThreads) {
+            if (nu_of<SM>(L)[k] != a) continue;
             const int64_t ma = gain_at<SM>(L, a, k);
 #pragma unroll
             for (int b = 0; b < DT; ++b)
@@ -932,54 +937,60 @@ __device__ __noinline__ void exchange_graph(const Layer& L, Team& tm, int lo) {
             }
     }
     team_sync(tm);
-    if (threadIdx.x < DMAX * DMAX)
-        sh.w[threadIdx.x / DMAX][threadIdx.x % DMAX] =
-            team_combine(wl + threadIdx.x, tm, [](uint64_t a, uint64_t b) { return a > b ? a : b; });
+    if (threadIdx.x < DMAX * DMAX) {
+        const int a = threadIdx.x / DMAX, b = threadIdx.x % DMAX;
+        if ((rows >> a) & 1u)
+            (lo < 0 ? sh.w : sh.wk)[a][b] =
+                team_combine(wl + threadIdx.x, tm, [](uint64_t a, uint64_t b) { return a > b ? a : b; });
+    }
     __syncthreads();
     tm.wph ^= 1;
 }
 
-// Thread 0 of every block: the best neuron of each edge of the path ending at `end` moves; each
-// block applies the moves of its own slice.
-template <bool SM>
-__device__ bool apply_path(const Layer& L, const int* pred, int end) {
-    Shared& sh = shared();
-    int v = end, steps = 0;
-    while (pred[v] >= 0) {
-        if (++steps > L.D) return false;
-        const int a = pred[v];
-        const int k = index_of(sh.w[a][v]) - L.k0;
-        if (k >= 0 && k < L.n) nu_of<SM>(L)[k] = static_cast<uint8_t>(v);
-        v = a;
+// Lane b: the gains of the edges into device b of an exchange graph (kNegInf: none).
+template <int DT>
+__device__ __forceinline__ void edges_into(const uint64_t (&graph)[DMAX][DMAX], int64_t (&w)[DT]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int a = 0; a < DT; ++a) {
+        const uint64_t e = lane < DT && lane != a ? graph[a][lane] : 0;
+        w[a] = e ? gain_of(e) : kNegInf;
     }
-    return true;
 }
 
-// Thread 0: max-gain path by Bellman-Ford over the D devices, from the devices
-// in `src` (dist 0) and relaxing the exchange graph sh.w.  Returns pred[].
-static __device__ __noinline__ void bellman_ford(const Layer& L, unsigned src, int64_t* dist, int* pred) {
+// Warp 0 of every block: the best neuron of each edge of the path ending at `end` moves (lane b holds
+// device b's predecessor on the path, -1 at its start); each block applies the moves of its own slice.
+// Returns the path's start, -1 if it has none; its devices go to sh.dirty.
+template <int DT, bool SM>
+__device__ __forceinline__ int apply_path(const Layer& L, const uint64_t (&graph)[DMAX][DMAX], int pred, int end) {
     Shared& sh = shared();
-    for (int a = 0; a < L.D; ++a) {
-        dist[a] = (src >> a) & 1u ? 0 : kNegInf;
-        pred[a] = -1;
-    }
-    for (int round = 0; round < L.D - 1; ++round)
-        for (int a = 0; a < L.D; ++a) {
-            if (dist[a] == kNegInf) continue;
-            for (int b = 0; b < L.D; ++b) {
-                if (b == a || sh.w[a][b] == 0) continue;
-                const int64_t nd = dist[a] + gain_of(sh.w[a][b]);
-                if (nd > dist[b]) dist[b] = nd, pred[b] = a;
-            }
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    unsigned touched = 0;
+    int v = end;
+    for (int steps = 0; steps < DT; ++steps) {        // a path visits a device once
+        touched |= 1u << v;
+        const int a = __shfl_sync(0xFFFFFFFFu, pred, v);
+        if (a < 0) {
+            if (lane0) sh.dirty = touched;
+            return v;
         }
+        const int k = index_of(graph[a][v]) - L.k0;
+        if (lane0 && k >= 0 && k < L.n) nu_of<SM>(L)[k] = static_cast<uint8_t>(v);
+        v = a;
+    }
+    return -1;
 }
 
 // Step (d) over all neurons.  assigned: L.nu is already optimal; else it is the assignment at some
-// prices and is balanced first.  The blocks of a team repeat the serial parts on equal data.
+// prices and is balanced first.  Warp 0 of every block of a team repeats the steps over the devices on
+// equal data.
 template <int DT, bool SM>
 __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned) {
     Shared& sh = shared();
     const int N = L.N, D = L.D, cap = L.cap;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) sh.dirty = (1u << DT) - 1u;
+    __syncthreads();
     if (!assigned) {
         for (int k = threadIdx.x; k < L.n; k += kThreads) atomicAdd(&sh.hist[tm.ph][kBins + nu_of<SM>(L)[k]], 1u);
         team_counters(tm);
@@ -991,24 +1002,25 @@ __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned)
             for (int l = 0; l < D; ++l) ex += sh.count[l] > cap ? 1 : 0;
             if (ex == 0) break;
             exchange_graph<DT, SM>(L, tm, -1);
-            if (threadIdx.x == 0) {
-                if (sh.beat && (aug & 31) == 31) atomicAdd(sh.beat, 1);
-                unsigned src = 0;
-                for (int l = 0; l < D; ++l)
-                    if (sh.count[l] > cap) src |= 1u << l;
-                int64_t dist[DMAX];
-                int pred[DMAX];
-                bellman_ford(L, src, dist, pred);
+            if (warp == 0) {
+                if (lane == 0 && sh.beat && (aug & 31) == 31) atomicAdd(sh.beat, 1);
+                const int cnt = lane < DT ? sh.count[lane] : cap;
+                const unsigned src = __ballot_sync(0xFFFFFFFFu, cnt > cap);
+                const unsigned snk = __ballot_sync(0xFFFFFFFFu, cnt < cap);
+                int64_t w[DT], dist;
+                int pred;
+                edges_into<DT>(sh.w, w);
+                bellman_ford_warp<DT>(src, w, dist, pred);
                 int e = -1;
-                for (int l = 0; l < D; ++l)
-                    if (sh.count[l] < cap && dist[l] != kNegInf && (e < 0 || dist[l] > dist[e])) e = l;
-                int s = e;
-                for (int steps = 0; e >= 0 && pred[s] >= 0 && steps <= D; ++steps) s = pred[s];
-                if (e < 0 || !apply_path<SM>(L, pred, e)) {
-                    sh.status = DTP_ERR_NOT_CONVERGED;
-                } else {
-                    sh.count[s] -= 1;
-                    sh.count[e] += 1;
+                int64_t best = kNegInf;
+                for (int b = 0; b < DT; ++b) {
+                    const int64_t x = __shfl_sync(0xFFFFFFFFu, dist, b);
+                    if (((snk >> b) & 1u) && x > best) best = x, e = b;
+                }
+                const int s = e < 0 ? -1 : apply_path<DT, SM>(L, sh.w, pred, e);
+                if (lane == 0) {
+                    if (s < 0) sh.status = DTP_ERR_NOT_CONVERGED;
+                    else sh.count[s] -= 1, sh.count[e] += 1;
                 }
             }
             __syncthreads();
@@ -1025,23 +1037,21 @@ __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned)
     int kstart = 0;
     for (int round = 0; round < N + 1; ++round) {
         exchange_graph<DT, SM>(L, tm, -1);
-        if (threadIdx.x == 0) {
-            if (sh.beat && (round & 31) == 31) atomicAdd(sh.beat, 1);
-            for (int a = 0; a < D; ++a)
-                for (int b = 0; b < D; ++b)
-                    sh.P[a][b] = (a == b) ? 0 : (sh.w[a][b] ? gain_of(sh.w[a][b]) : kNegInf);
-            for (int c = 0; c < D; ++c)
-                for (int a = 0; a < D; ++a)
-                    for (int b = 0; b < D; ++b)
-                        if (sh.P[a][c] != kNegInf && sh.P[c][b] != kNegInf && sh.P[a][c] + sh.P[c][b] > sh.P[a][b])
-                            sh.P[a][b] = sh.P[a][c] + sh.P[c][b];
-            for (int a = 0; a < D; ++a)
-                if (sh.P[a][a] > 0) sh.status = DTP_ERR_NOT_CONVERGED;  // a positive cycle: not optimal
-            // prices for the next neuron step: longest paths from a zero root
-            for (int a = 0; a < D; ++a) sh.pi[a] = 0;
-            for (int a = 0; a < D; ++a)
-                for (int b = 0; b < D; ++b)
-                    if (sh.P[a][b] != kNegInf && sh.P[a][b] > sh.pi[b]) sh.pi[b] = sh.P[a][b];
+        if (warp == 0) {
+            if (lane == 0 && sh.beat && (round & 31) == 31) atomicAdd(sh.beat, 1);
+            for (int i = lane; i < DT * DT; i += 32) {
+                const int a = i / DT, b = i % DT;
+                sh.P[a][b] = a == b ? 0 : (sh.w[a][b] ? gain_of(sh.w[a][b]) : kNegInf);
+            }
+            __syncwarp();
+            close_paths(DT);
+            if (lane < DT) {
+                if (sh.P[lane][lane] > 0) sh.status = DTP_ERR_NOT_CONVERGED;   // a positive cycle: not optimal
+                // prices for the next neuron step: longest paths from a zero root
+                int64_t pot = 0;
+                for (int a = 0; a < DT; ++a) pot = sh.P[a][lane] > pot ? sh.P[a][lane] : pot;
+                sh.pi[lane] = pot;
+            }
         }
         __syncthreads();
         if (sh.status != DTP_OK) return;
@@ -1069,18 +1079,20 @@ __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned)
                 !own ? 0 : (threadIdx.x < DT ? gain_at<SM>(L, threadIdx.x, k) : static_cast<int64_t>(nu_of<SM>(L)[k]));
         }
         team_sum_i64(DT + 1, tm);
-        if (threadIdx.x == 0) {
+        if (warp == 0) {
             const int t = static_cast<int>(sh.B[DT]);
+            int64_t w[DT], dist;
+            int pred;
+            edges_into<DT>(sh.wk, w);
+            if (lane == 0) sh.dirty = 0;
             for (int l = 0; l < t; ++l) {
-                int64_t dist[DMAX];
-                int pred[DMAX];
-                bellman_ford(L, 1u << l, dist, pred);
-                if (dist[t] != kNegInf && sh.B[l] - sh.B[t] + dist[t] == 0) {
-                    if (!apply_path<SM>(L, pred, t)) sh.status = DTP_ERR_NOT_CONVERGED;
-                    const int k = kstar - L.k0;
-                    if (k >= 0 && k < L.n) nu_of<SM>(L)[k] = static_cast<uint8_t>(l);
-                    break;
-                }
+                bellman_ford_warp<DT>(1u << l, w, dist, pred);
+                const int64_t to = __shfl_sync(0xFFFFFFFFu, dist, t);
+                if (to == kNegInf || sh.B[l] - sh.B[t] + to != 0) continue;
+                if (apply_path<DT, SM>(L, sh.wk, pred, t) < 0 && lane == 0) sh.status = DTP_ERR_NOT_CONVERGED;
+                const int k = kstar - L.k0;
+                if (lane == 0 && k >= 0 && k < L.n) nu_of<SM>(L)[k] = static_cast<uint8_t>(l);
+                break;
             }
         }
         __syncthreads();
