@@ -149,7 +149,8 @@ int64_t partition_count(int G, int D) {
 }
 
 // Workspace of a layer that may have to live in global memory (where no cluster can hold it): int64
-// gains, int32 labels and N more words, which cover slice_bytes(N, D).
+// gains, int32 labels and N more words, which cover the slices of any team (slice_bytes: 2 D + 11 bytes a
+// neuron fewer, against 16 neurons and 256 bytes a block of rounding, on more than 3000 neurons).
 static size_t global_layer_bytes(int N, int D) {
     return align_up(static_cast<size_t>(N) * D * sizeof(int64_t) + static_cast<size_t>(N) * sizeof(int32_t), 256) +
            align_up(static_cast<size_t>(N) * sizeof(uint64_t), 256);
@@ -163,7 +164,7 @@ static bool fits_block(int N, int D) {
 
 struct Plan {
     int cl;        // blocks per team
-    int global;    // 1: cl == 1 and the layer lives in the workspace
+    int global;    // 1: the layer lives in the workspace
     size_t dyn;
     View vw;
 };
@@ -209,7 +210,10 @@ static int resident_teams(int dev, int cl) {
 // and 52, but beside the affinity pass four blocks cost 1% of a step and two nothing).  A larger layer
 // takes as few blocks as hold it, then up to 8 (the portable cluster size) while a block has more than
 // kSliceTarget neurons and every team has its SMs to itself (N = 14336, D = 8: 4.5 ms in one block with
-// the layer in global memory, 0.25 ms in 8).
+// the layer in global memory, 0.25 ms in 8).  A layer too large for that lives in the workspace and takes
+// the largest team, or 8 blocks where such teams run one after another: its passes wait for L2, and fewer
+// layers at a time stay there (N = 262144, D = 2: one layer 5.6 ms in one block, 0.26 in 16; 160 layers
+// 10.8 ms in a block each, 6.3 in teams of 8).
 constexpr int kSliceTarget = 1024, kGatheredTarget = 768;
 static int make_plan(int64_t teams, int rows, int N, int D, Plan* p) {
     int dev = 0, sms = 0;
@@ -221,11 +225,13 @@ static int make_plan(int64_t teams, int rows, int N, int D, Plan* p) {
     while (cl < kMaxCluster && slice_bytes(slice_np(N, cl), D) > kSmemBudget) cl *= 2;
     if (cl > most || slice_bytes(slice_np(N, cl), D) > kSmemBudget) {
         if (fits_block(N, D)) return DTP_ERR_WORKSPACE;   // no room was asked for: never with the budgets above
-        p->cl = 1;
+        cl = most > 8 && teams > resident_teams(dev, most) ? 8 : most;
+        if (cl * align_up(slice_bytes(slice_np(N, cl), D), 256) > global_layer_bytes(N, D)) return DTP_ERR_WORKSPACE;
+        p->cl = cl;
         p->global = 1;
         p->dyn = 0;
-        p->vw.np = slice_np(N, 1);
-        p->vw.gathered = 1;
+        p->vw.np = slice_np(N, cl);
+        p->vw.gathered = cl == 1;
         p->vw.rows = 0;
         return DTP_OK;
     }

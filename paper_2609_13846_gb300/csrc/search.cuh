@@ -3,8 +3,8 @@
 // neuron assignments nu of one layer, maximising the co-located up-edge mass.
 //
 // One team per layer: a thread block cluster of 1 to 16 blocks of 512 threads,
-// each holding a slice of the layer's neurons in shared memory (a single block
-// with the layer in global memory when even 16 slices do not fit).  Each block
+// each holding a slice of the layer's neurons in shared memory (in global
+// memory when even 16 slices do not fit).  Each block
 // reduces its slice, one cluster barrier later every block reads its peers'
 // partial results over distributed shared memory and continues with the same
 // totals, so the serial parts are repeated by every block instead of broadcast.
@@ -1414,17 +1414,18 @@ __device__ __forceinline__ void neuron_step(const Layer& L, Team& tm) {
 // sh.xl[phase][r * DT + l] = the slice's sum of score row r over its neurons on device l, for rows
 // r < rows; nu: the slice's labels.  The neurons are first listed by device (over the gains, which the
 // next step rebuilds),
-// then a power of two of threads adds each (row, device) list: 2.5 times fewer instructions than
-// walking every row with a select per device.
+// then a power of two of threads adds each (row, device) list (several warps where there are few
+// lists): 2.5 times fewer instructions than walking every row with a select per device.
 template <int DT, bool SM>
 __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, Team& tm, int rows) {
     Shared& sh = shared();
     const Layer L = layer;
     const int tid = threadIdx.x, lane = tid & 31;
     uint16_t* lists = SM ? reinterpret_cast<uint16_t*>(dsm + kData) : L.lists;
-    const bool wide = L.rnp > 65535;                            // a layer in global memory: 32-bit indices
+    const bool wide = L.rnp > 65535;            // 32-bit indices: only where no cluster of four can be resident
     uint32_t* lists32 = reinterpret_cast<uint32_t*>(lists);
     if (tid < DMAX) sh.clen[tid] = 0;
+    if (tid < rows * DT) sh.xl[tm.lph][tid] = 0;
     __syncthreads();
     for (int k0 = 0; k0 < L.n; k0 += kThreads) {
         const int k = k0 + tid;
@@ -1439,27 +1440,45 @@ __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, 
         }
     }
     __syncthreads();
-    const int pairs = rows * DT;                                // at most 256
-    int tpp = 32;
-    while (tpp * pairs > kThreads) tpp >>= 1;
-    for (int i = tid; i < pairs * tpp; i += kThreads) {         // whole groups of tpp lanes
-        const int pair = i / tpp, sub = i % tpp;
+    const int pairs = rows * DT;                                // 4 to 256
+    int tpp = kThreads / 4;
+    while (tpp * pairs > kThreads) tpp >>= 1;                   // 2 to 128
+    if (tid < pairs * tpp) {                                    // whole groups of tpp lanes, or whole warps
+        const int pair = tid / tpp, sub = tid % tpp;
         const int r = pair / DT, l = pair % DT;
         const int len = sh.clen[l];
         int64_t hs = 0;
         uint32_t ls = 0;
-        for (int j = sub; j < len; j += tpp) {
-            const int k = wide ? static_cast<int>(lists32[l * L.rnp + j]) : lists[l * L.rnp + j];
+        auto entry = [&](int j) -> int {
+            return wide ? static_cast<int>(lists32[l * L.rnp + j]) : lists[l * L.rnp + j];
+        };
+        int j = sub;
+        for (; j + 3 * tpp < len; j += 4 * tpp) {               // four neurons' loads in flight
+            int k[4];
+            uint32_t h[4], lo[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) k[u] = entry(j + u * tpp);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) score_parts<SM>(L, r, k[u], h[u], lo[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) hs += h[u], ls += lo[u];
+        }
+        for (; j < len; j += tpp) {
             uint32_t h, lo;
-            score_parts<SM>(L, r, k, h, lo);
+            score_parts<SM>(L, r, entry(j), h, lo);
             hs += h;
             ls += lo;
         }
         // the group's own lanes: their lists differ in length, so they need not leave the loop together
-        const unsigned group = (0xFFFFFFFFu >> (32 - tpp)) << (lane & ~(tpp - 1));
+        const int width = tpp < 32 ? tpp : 32;
+        const unsigned group = (0xFFFFFFFFu >> (32 - width)) << (lane & ~(width - 1));
         int64_t v = (hs << kLoBits) + ls;
-        for (int o = tpp >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(group, v, o);
-        if (sub == 0) sh.xl[tm.lph][pair] = v;
+        for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(group, v, o);
+        if (tpp <= 32) {
+            if (sub == 0) sh.xl[tm.lph][pair] = v;
+        } else if (lane == 0) {
+            atomicAdd(reinterpret_cast<unsigned long long*>(&sh.xl[tm.lph][pair]), static_cast<unsigned long long>(v));
+        }
     }
 }
 
@@ -1556,7 +1575,15 @@ struct View {
 
 __host__ __device__ inline int gains_np(const View& vw, int N) { return vw.gathered ? (N + 15) / 16 * 16 : vw.np; }
 
-// This block's part, over buf (shared memory, or global memory for a team of one block).
+// Where a block's slice lies: in shared memory, or in the team's buffer of `per_team` bytes.
+template <bool SM>
+__device__ __forceinline__ uint8_t* slice_buf(uint8_t* gbuf, int64_t team, size_t per_team, const View& vw, int D,
+                                              const Team& tm) {
+    if constexpr (SM) return dsm + kData;
+    else return gbuf + static_cast<size_t>(team) * per_team + tm.rank * align_up_dev(slice_bytes(vw.np, D), 256);
+}
+
+// This block's part, over buf.
 static __device__ void layer_view(Layer& L, int G, int N, int D, uint8_t* buf, const View& vw, const Team& tm) {
     L.G = G;
     L.N = N;
@@ -1699,7 +1726,7 @@ search_kernel(const float* __restrict__ A_all, int G, int N, int iters, int32_t*
     Shared& sh = shared();
     Team tm = make_team();
     const int layer = blockIdx.x / tm.cl;
-    uint8_t* buf = SM ? dsm + kData : gbuf + static_cast<size_t>(layer) * per_layer;
+    uint8_t* buf = slice_buf<SM>(gbuf, layer, per_layer, vw, DT, tm);
     Layer L;
     layer_view(L, G, N, DT, buf, vw, tm);
     init_shared();
@@ -1855,11 +1882,11 @@ template <int DT, bool SM>
 __global__ void __launch_bounds__(kThreads, 1)
 global_items_kernel(const float* __restrict__ A_all, int layers, int G, int N, int64_t n_unl,
                     int64_t* __restrict__ values, int* __restrict__ ws_status, uint8_t* __restrict__ gbuf,
-                    size_t per_block, View vw) {
+                    size_t per_team, View vw) {
     Shared& sh = shared();
     Team tm = make_team();
     const int64_t team = blockIdx.x / tm.cl, teams = gridDim.x / tm.cl;
-    uint8_t* buf = SM ? dsm + kData : gbuf + static_cast<size_t>(blockIdx.x) * per_block;
+    uint8_t* buf = slice_buf<SM>(gbuf, team, per_team, vw, DT, tm);
     const int64_t items = static_cast<int64_t>(layers) * n_unl;
     Team own = make_own(tm);
     init_shared();
@@ -1912,7 +1939,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 global_pick_kernel(const float* __restrict__ A_all, int G, int N, int64_t n_unl, const int64_t* __restrict__ values,
                    int32_t* __restrict__ head_out, int32_t* __restrict__ nu_out, int64_t* __restrict__ score_q_out,
                    double* __restrict__ score_out, int* __restrict__ ws_status, uint8_t* __restrict__ gbuf,
-                   size_t per_block, View vw) {
+                   size_t per_team, View vw) {
     Shared& sh = shared();
     Team tm = make_team();
     const int layer = blockIdx.x / tm.cl;
@@ -1950,7 +1977,7 @@ global_pick_kernel(const float* __restrict__ A_all, int G, int N, int64_t n_unl,
         if (threadIdx.x == 0) atomicMin(ws_status, static_cast<int>(DTP_ERR_ARG));
         return;
     }
-    uint8_t* buf = SM ? dsm + kData : gbuf + static_cast<size_t>(layer) * per_block;
+    uint8_t* buf = slice_buf<SM>(gbuf, layer, per_team, vw, DT, tm);
     Layer L;
     layer_view(L, G, N, DT, buf, vw, tm);
     set_partition(sh.best_idx, G, DT);
@@ -2153,7 +2180,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_iteration_kernel(const Chai
     const int i = blockIdx.x / tm.cl;
     const int G = c.G, N = c.N, tid = threadIdx.x;
     const int64_t GN = static_cast<int64_t>(G) * N;
-    uint8_t* buf = SM ? dsm + kData : c.gbuf + static_cast<size_t>(i) * c.per_layer;
+    uint8_t* buf = slice_buf<SM>(c.gbuf, i, c.per_layer, c.vw, DT, tm);
     Layer L;
     layer_view(L, G, N, DT, buf, c.vw, tm);
     init_shared();

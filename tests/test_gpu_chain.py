@@ -86,16 +86,16 @@ def test_chain_captured_in_a_graph():
             assert torch.equal(got[k], want[k])
 
 
-@pytest.mark.parametrize("G,N,D", WIDEST)
-def test_chain_widest_layers(G, N, D):
-    """One iteration on three layers: certified neuron steps, the oracle's head steps and score on them."""
-    Su, Sd = _model(3, G, N, seed=N)
+@pytest.mark.parametrize("L,G,N,D", [(3, *w) for w in WIDEST] + [(20, 8, 65544, 8)])
+def test_chain_widest_layers(L, G, N, D):
+    """One iteration on three layers, and on more than there are teams at once: certified neuron steps, the oracle's head steps and score on them."""
+    Su, Sd = _model(L, G, N, seed=N)
     up, down = [oracle.normalize_unit_mass(S) for S in Su], [oracle.normalize_unit_mass(S) for S in Sd]
     h0 = np.arange(G) * D // G
     r = dtp.search_chain(torch.as_tensor(Su, device=DEV), torch.as_tensor(Sd, device=DEV), D, 1)
     h, nu = r["h"].cpu().numpy(), r["nu"].cpu().numpy()
-    for i in range(3):
-        gain = up[i] + down[i] if i < 2 else up[i]
+    for i in range(L):
+        gain = up[i] + down[i] if i < L - 1 else up[i]
         assert only_optimum(np.stack([gain[h0 == l].sum(axis=0) for l in range(D)], axis=1), nu[i])
         fed = [(up[i], nu[i])] + ([(down[i - 1], nu[i - 1])] if i > 0 else [])
         want, _ = oracle.head_step(np.concatenate([f[0] for f in fed], axis=1), np.concatenate([f[1] for f in fed]), D)

@@ -106,7 +106,7 @@ def only_optimum(M, nu):
     return bool((np.diagonal(w) < 0).all())
 
 
-# 16 blocks, then gains in global memory: with 16-bit lists of neurons, and with 32-bit ones
+# 16 blocks; beyond what they hold, gains in global memory
 WIDEST = [(8, 40000, 8), (8, 61448, 8), (8, 65544, 8), (4, 120580, 4)]
 
 
@@ -129,6 +129,16 @@ def test_widest_layers(G, N, D):
         np.testing.assert_array_equal(g["h"].cpu().numpy(), h0)
         np.testing.assert_array_equal(g["nu"].cpu().numpy(), nu)
         assert int(g["score_q"]) == oracle.layout_score(q, h0, nu)
+
+
+def test_widest_layers_batched():
+    """More layers in global memory than teams of 16 blocks at once: each as by itself."""
+    As = torch.stack([synth.make_affinity_matrix(8, 65544, seed=i) for i in range(3)]).to(DEV)
+    one = [dtp.search_layout(A, 8, 2) for A in As]
+    r = dtp.search_layout_batched(As.repeat(10, 1, 1).contiguous(), 8, 2)
+    for i in range(30):
+        for k in r:
+            assert torch.equal(r[k][i], one[i % 3][k].reshape(r[k][i].shape)), k
 
 
 def test_full_size_llama_neuron_count_d8():
