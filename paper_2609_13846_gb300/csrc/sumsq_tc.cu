@@ -425,28 +425,40 @@ __global__ void sumsq_reduce_kernel(const float* __restrict__ partial, float* __
 }
 
 // WdT[k, i] = bf16(gamma[i] * W_down[i, k]): gamma' . w^d_k as K-major rows.  Bound by reading W_down and
-// writing WdT once: 64 x 64 tiles, 16-byte writes along i and (kWide: rows on 16-byte boundaries) 16-byte
-// reads along k.  1024 x 3072: 9.3 us with 32 x 32 tiles of single elements, 5.8 us now.
-constexpr int kPrepTile = 64;
+// writing WdT once, small ones by the latency of a block: 16-byte writes along i, and with rows on 16-byte
+// boundaries (kWide) 16-byte reads along k in 64 x 64 tiles (1024 x 3072: 5.2 us, 8.6 with single elements
+// both ways).
+// Other rows take 32 x 32 tiles of single reads: 88 x 773 2.1 us, 288 x 126 2.1, 1024 x 3001 6.7, 4096 x
+// 14337 84 (in 64 x 64 tiles 3.4, 3.4, 6.2 and 75; with single writes too 2.4, 2.3, 8.4 and 124).
+template <bool kWide>
+constexpr int kPrepTileOf = kWide ? 64 : 32;
 template <bool kWide>
 __global__ void __launch_bounds__(256)
 prep_down_weight_kernel(const __nv_bfloat16* __restrict__ Wd, const __nv_bfloat16* __restrict__ gamma, int d, int N,
                         __nv_bfloat16* __restrict__ WdT) {
+    constexpr int kPrepTile = kPrepTileOf<kWide>;
     __shared__ __nv_bfloat16 tile[kPrepTile][kPrepTile + 2];   // [i][k]
     const int i0 = blockIdx.y * kPrepTile, k0 = blockIdx.x * kPrepTile;
     constexpr int kPer = kWide ? 8 : 1;
-    for (int x = threadIdx.x; x < kPrepTile * kPrepTile / kPer; x += 256) {
-        const int r = x / (kPrepTile / kPer), c = x % (kPrepTile / kPer) * kPer;
-        const int i = i0 + r, k = k0 + c;
-        if (i >= d || k >= N) continue;                        // kWide: N is a multiple of 8
-        const float g = static_cast<float>(gamma[i]);
-        union { uint4 q; __nv_bfloat16 e[8]; } w;
-        const __nv_bfloat16* src = Wd + static_cast<int64_t>(i) * N + k;
-        if constexpr (kWide) w.q = *reinterpret_cast<const uint4*>(src);
-        else w.e[0] = *src;
+    constexpr int kLoads = kPrepTile * kPrepTile / kPer / 256;  // per thread, all in flight
+    constexpr int kStep = 256 / (kPrepTile / kPer);             // rows apart
+    const int r0 = threadIdx.x / (kPrepTile / kPer), c = threadIdx.x % (kPrepTile / kPer) * kPer;
+    union { uint4 q; __nv_bfloat16 e[8]; } w[kLoads];
+    float g[kLoads];
+    const int k = min(k0 + c, N - kPer);                        // beyond the edges: values that nothing reads
 #pragma unroll
-        for (int v = 0; v < kPer; ++v) tile[r][c + v] = __float2bfloat16_rn(g * static_cast<float>(w.e[v]));
+    for (int j = 0; j < kLoads; ++j) {
+        const int i = min(i0 + r0 + j * kStep, d - 1);
+        const __nv_bfloat16* src = Wd + static_cast<int64_t>(i) * N + k;
+        g[j] = static_cast<float>(__ldg(gamma + i));
+        if constexpr (kWide) w[j].q = __ldg(reinterpret_cast<const uint4*>(src));   // N is a multiple of 8
+        else w[j].e[0] = __ldg(src);
     }
+#pragma unroll
+    for (int j = 0; j < kLoads; ++j)
+#pragma unroll
+        for (int v = 0; v < kPer; ++v)
+            tile[r0 + j * kStep][c + v] = __float2bfloat16_rn(g[j] * static_cast<float>(w[j].e[v]));
     __syncthreads();
     for (int x = threadIdx.x; x < kPrepTile * (kPrepTile / 8); x += 256) {
         const int c = x % kPrepTile, r = x / kPrepTile * 8;    // column k0 + c, rows i0 + r .. + 7 (d % 8 == 0)
@@ -560,8 +572,10 @@ int launch_down(const void* Wqkv, const void* gamma, const void* Wd, int G, int 
     __nv_bfloat16* WdT = reinterpret_cast<__nv_bfloat16*>(ws + kWorkspaceHeader);
     float* partial = reinterpret_cast<float*>(ws + kWorkspaceHeader + align_up(static_cast<size_t>(N) * d * 2, 256));
     if (dtype != DTP_BF16) return DTP_ERR_UNSUPPORTED;
-    const dim3 pg((N + kPrepTile - 1) / kPrepTile, (d + kPrepTile - 1) / kPrepTile);
-    auto* prep = N % 8 == 0 ? prep_down_weight_kernel<true> : prep_down_weight_kernel<false>;   // Wd is 16-byte aligned
+    const bool wide = N % 8 == 0;                               // Wd is 16-byte aligned
+    const int tile = wide ? kPrepTileOf<true> : kPrepTileOf<false>;
+    const dim3 pg((N + tile - 1) / tile, (d + tile - 1) / tile);
+    auto* prep = wide ? prep_down_weight_kernel<true> : prep_down_weight_kernel<false>;
     prep<<<pg, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(Wd), static_cast<const __nv_bfloat16*>(gamma), d, N,
                                  WdT);
     DTP_CUDA_TRY(cudaGetLastError());

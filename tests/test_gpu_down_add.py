@@ -129,6 +129,12 @@ def test_down_sqnorm_sizes(d, N, dtype):
     assert torch.all((got - want).abs() <= max(d, 4) * 2.0 ** -24 * want)
 
 
+@pytest.mark.parametrize("G,R,d,N", [(2, 33, 8, 1), (1, 16, 40, 33), (3, 70, 104, 31), (2, 64, 64, 97), (1, 48, 200, 72)])
+def test_down_weight_tile_edges(G, R, d, N):
+    """W_down transposed in tiles: rows on odd boundaries (32 x 32 tiles) and of whole 16-byte words (64 x 64)."""
+    test_down_weight_sqnorm(G, R, d, N)
+
+
 def test_down_weight_sqnorm_beyond_half_of_l2():
     """gamma' . W_down^T of 128 MiB (d = 4096, N = 16384): single CTAs; two whole column tiles and
     sampled columns (column k of ||b_gk||^2 depends only on column k of W_down)."""
