@@ -129,6 +129,13 @@ def test_down_sqnorm_sizes(d, N, dtype):
     assert torch.all((got - want).abs() <= max(d, 4) * 2.0 ** -24 * want)
 
 
+@pytest.mark.parametrize("d,N", [(3, 40000), (70, 38916), (9, 80000), (20, 77832)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_down_sqnorm_wide(d, N, dtype):
+    """Wide enough for 32 lanes a row (N from 38912 fp32, 77824 bf16 on 152 SMs), the last block ragged."""
+    test_down_sqnorm_sizes(d, N, dtype)
+
+
 @pytest.mark.parametrize("G,R,d,N", [(2, 33, 8, 1), (1, 16, 40, 33), (3, 70, 104, 31), (2, 64, 64, 97), (1, 48, 200, 72)])
 def test_down_weight_tile_edges(G, R, d, N):
     """W_down transposed in tiles: rows on odd boundaries (32 x 32 tiles) and of whole 16-byte words (64 x 64)."""
