@@ -124,9 +124,10 @@ def test_apply_layout_bit_exact(d, Hq, G, hd, N, D):
         assert torch.equal(out[k].cpu().float(), torch.as_tensor(ref[k], dtype=torch.float32)), k
 
 
-@pytest.mark.parametrize("layers,n,D", [(2, 1025, 5), (1, 65528, 8), (1, 65544, 8), (2, 99, 9), (1, 7, 1)])
+@pytest.mark.parametrize("layers,n,D", [(2, 1025, 5), (1, 65528, 8), (1, 65544, 8), (2, 99, 9), (1, 7, 1),
+                                        (2, 65541, 3), (1, 131072, 2), (1, 65600, 16)])
 def test_layout_order_scan_forms(layers, n, D):
-    """All devices' counts in one packed scan (D <= 8, n <= 65535) and device by device beyond."""
+    """All devices' counts in one packed scan (D <= 8; 16 bits up to n = 65535, 32 beyond), else device by device."""
     test_layout_order_bit_exact(layers, n, D)
 
 
