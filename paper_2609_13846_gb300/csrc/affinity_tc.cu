@@ -730,13 +730,17 @@ static int64_t busiest_passes(int64_t units, int64_t workers, int G) {
 // (each SM has the same multiply-adds to do) and is 12% faster in fact: it keeps the tensor pipe 97% busy,
 // a single CTA 87%.  But single CTAs have twice the units of half the tokens to spread over the chip, which
 // wins on short inputs: 777 tokens of a Qwen-shaped layer run 11 single passes against 13 in pairs (69 us
-// against 72), 128 tokens 3 against 4.
-static bool prefer_pairs(int NT, int TC, int G, int cap, int resident) {
+// against 72), 128 tokens 3 against 4.  Weights that fill L2 nearly to the half where chunk grouping begins
+// make a single's pass 20 to 28% slower (each reads the weights from L2 for itself): 777 tokens, d = 2048,
+// N = 8192, 4 heads, 15 passes against 18: 202 us against 191; 600 tokens, 8 heads, 20 against 27: 263
+// against 271.  Beyond, with grouping, it is 10 to 16% again (d = 4096, N = 14336, 600 tokens, 36 passes
+// against 41: 828 us against 873; 1300 tokens, 74 against 81: 1764 against 1705).
+static bool prefer_pairs(int NT, int TC, int G, int cap, int resident, bool filling) {
     int64_t pairs = cap / 2 < resident ? cap / 2 : resident;
     if (pairs < 1) pairs = 1;
     const int64_t in_pairs = busiest_passes(static_cast<int64_t>(NT) * ((TC + 1) / 2), pairs, G);
     const int64_t in_singles = busiest_passes(static_cast<int64_t>(NT) * TC, cap, G);
-    return 100 * in_pairs <= 112 * in_singles;
+    return 100 * in_pairs <= (filling ? 124 : 112) * in_singles;
 }
 
 // G heads of C; A receives G / qpg rows (qpg consecutive heads summed per row).  max_ctas > 0
@@ -769,7 +773,8 @@ int launch_grouped(const void* X, const void* C, const void* Wg, const void* Wu,
     DTP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     DTP_CUDA_TRY(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
     const double tile_bytes = 2.0 * BNEU * d * 2.0;   // W_gate and W_up rows of one neuron tile
-    const bool weights_fit = static_cast<double>(p.NT) * tile_bytes <= l2 / 2.0;
+    const double weights = static_cast<double>(p.NT) * tile_bytes;
+    const bool weights_fit = weights <= l2 / 2.0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -797,7 +802,8 @@ int launch_grouped(const void* X, const void* C, const void* Wg, const void* Wu,
     }
     const int cap = (max_ctas > 0 && max_ctas < sms) ? max_ctas : sms;
     const bool pair = resident > 0 && (cap >= 2 || weights_fit) &&
-                      prefer_pairs(p.NT, static_cast<int>((T + BT - 1) / BT), G, cap, resident);
+                      prefer_pairs(p.NT, static_cast<int>((T + BT - 1) / BT), G, cap, resident,
+                                   weights_fit && weights > 0.375 * l2);
     auto kernel = pair ? affinity_fo_tc_kernel<true> : affinity_fo_tc_kernel<false>;
     const size_t smem = pair ? Form<true>::kSmemBytes : Form<false>::kSmemBytes;
     DTP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));

@@ -231,6 +231,17 @@ def test_weights_beyond_half_of_l2(T, max_ctas):
     assert _rel_fro(got, ref) <= BF16_TOL
 
 
+@pytest.mark.parametrize("G,T", [(8, 600), (4, 777)])   # 27 pair passes against 20 single ones, 18 against 15
+def test_short_inputs_on_weights_that_nearly_fill_half_of_l2(G, T):
+    """W_gate + W_up of 64 MiB (d = 2048, N = 8192): single CTAs only where they save a quarter of the passes."""
+    d, N = 2048, 8192
+    L = synth.make_layer(d, G, N, T, seed=62, dtype="bf16")
+    A = dtp.affinity_accumulate(*(L[k].to(DEV) for k in ("X", "C", "W_gate", "W_up")))
+    cols = np.unique(np.concatenate([np.random.default_rng(2).choice(N, size=5, replace=False), [0, 127, 128, N - 1]]))
+    got = A[:, torch.as_tensor(cols, device=DEV)].double().cpu().numpy()
+    assert _rel_fro(got, _oracle(L, rows=cols)) <= BF16_TOL
+
+
 @pytest.mark.parametrize("T", [6145, 12500])   # two and three launches, the last ragged; up to 6143 one
 def test_long_input_on_weights_beyond_l2_runs_in_launches(T):
     """One call on more tokens than a launch takes equals the same tokens streamed in two calls, for both
