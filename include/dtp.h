@@ -117,13 +117,15 @@ int dtp_affinity_accumulate_ex(const void* X, const void* C, const void* W_gate,
 /*
  * Launch options of the bf16 affinity pass.
  *   max_ctas   0: one persistent CTA per SM (the default of the other entry
- *              points); n > 0: at most n CTAs, leaving the other SMs to
- *              kernels running concurrently on other streams (for instance the
- *              layout search of the previous layer, which runs on two SMs when the layer's
- *              gains fit in one block's shared memory, else on up to 16).
- *              The kernel usually runs as pairs of CTAs, and n is then rounded
- *              down to an even count (when the layer's W_gate and W_up fit in
- *              half of the L2 cache: at least one pair, 2 CTAs for n = 1)
+ *              points); n > 0: at most n CTAs, rounded down to an even count
+ *              (n = 1: one CTA, or one pair where the kernel runs as pairs of
+ *              CTAs and W_gate and W_up fit in half of the L2 cache), leaving
+ *              the other SMs to kernels running concurrently on other
+ *              streams.  n = SMs - 1 leaves two, enough for
+ *              dtp_search_layout on a layer whose gains fit in one block's
+ *              shared memory (one or two blocks).  The search of a larger
+ *              layer, of several at once and of a whole model takes more
+ *              blocks, in clusters of up to 16, and starts as the pass ends
  *   flags      DTP_AFFINITY_DEFER_REDUCE: launch only the main kernel; its
  *              per-unit partial sums stay in the workspace and
  *              dtp_affinity_reduce adds them into A (and act2) later, possibly

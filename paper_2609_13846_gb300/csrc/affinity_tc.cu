@@ -800,7 +800,10 @@ int launch_grouped(const void* X, const void* C, const void* Wg, const void* Wu,
         }
         if (dev < 64) resident_cache[dev].store(resident, std::memory_order_relaxed);
     }
-    const int cap = (max_ctas > 0 && max_ctas < sms) ? max_ctas : sms;
+    // a cap rounds down to an even count in both forms: what it leaves then holds a cluster of two (777 tokens,
+    // d = 4096, N = 3072 in 151 single CTAs: the layout search beside them ended with the pass, at 255 us;
+    // in 150 at 138)
+    const int cap = (max_ctas > 0 && max_ctas < sms) ? (max_ctas > 1 ? max_ctas & ~1 : 1) : sms;
     const bool pair = resident > 0 && (cap >= 2 || weights_fit) &&
                       prefer_pairs(p.NT, static_cast<int>((T + BT - 1) / BT), G, cap, resident,
                                    weights_fit && weights > 0.375 * l2);

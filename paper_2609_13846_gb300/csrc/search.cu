@@ -205,7 +205,7 @@ static int resident_teams(int dev, int cl) {
 
 // Blocks per team for `teams` layers of `rows` score rows at once.  A layer that fits in one block is
 // gathered there and the other blocks build gains and sum columns: one layer alone takes two blocks,
-// which a pass capped at one SM less than the chip leaves free in its pair form (28 Qwen-shaped layers,
+// which a pass capped at one SM less than the chip leaves free (it rounds down; 28 Qwen-shaped layers,
 // D = 4, whole model: 493 us with one block each, 415 with two, 354 with four; one layer, D = 2: 76, 60
 // and 52, but beside the affinity pass four blocks cost 1% of a step and two nothing).  A larger layer
 // takes as few blocks as hold it, then up to 8 (the portable cluster size) while a block has more than

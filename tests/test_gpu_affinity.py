@@ -260,6 +260,32 @@ def test_long_input_on_weights_beyond_l2_runs_in_launches(T):
     assert torch.equal(capped, A)
 
 
+@pytest.mark.parametrize("T", [777, 2048])   # single CTAs, CTA pairs
+def test_search_runs_beside_a_pass_capped_below_the_chip(T):
+    """A pass capped at one SM less than the chip leaves room for the search of a layer that one block holds
+    (two blocks): queued after the pass has started, the search ends well before it."""
+    d, G, N = 3072, 16, 3072
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    L = synth.make_layer(d, G, N, T, seed=63, dtype="bf16", device=DEV)
+    A, ws = torch.zeros(G, N, device=DEV), dtp.affinity_workspace(T, d, G, N, dtp.DTP_BF16, DEV)
+    S = synth.make_affinity_matrix(8, N, seed=64).to(DEV)
+    ws_s = torch.empty(dtp.search_workspace_size(1, 8, N, 2), dtype=torch.uint8, device=DEV)
+    main, side = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    lead = []
+    for _ in range(6):
+        begin, end, found = (torch.cuda.Event(enable_timing=True) for _ in range(3))
+        with torch.cuda.stream(main):
+            begin.record(main)
+            dtp.affinity_accumulate(L["X"], L["C"], L["W_gate"], L["W_up"], A=A, workspace=ws, max_ctas=n_sms - 1)
+            end.record(main)
+        dtp.search_layout(S, 2, 10, workspace=ws_s, stream=side, check=False)
+        found.record(side)
+        torch.cuda.synchronize()
+        lead.append(found.elapsed_time(end) / begin.elapsed_time(end))
+    assert sorted(lead)[3] > 0.25      # 0 where the search has to wait for the pass
+
+
 @pytest.mark.parametrize("max_ctas", [1, 7, 151])
 def test_grid_cap_does_not_change_the_result(max_ctas):
     """The persistent grid may be capped (SMs left to a concurrent search); A is bitwise the same."""
