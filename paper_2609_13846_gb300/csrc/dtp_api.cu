@@ -26,7 +26,7 @@ int launch_grouped(const float* X, const float* C, const float* Wg, const float*
 }  // namespace f32
 namespace sq {
 size_t down_workspace_bytes(int G, int R, int d, int N);
-int launch_down(const void* Wqkv, const void* gamma, const void* Wd, int G, int R, int d, int N, int dtype, float* bn,
+int launch_down(const void* Wqkv, const void* gamma, const void* Wd, int G, int R, int d, int N, float* bn,
                 void* workspace, cudaStream_t stream);
 size_t add_workspace_bytes(int64_t T, int G, int N);
 int launch_add(const void* C, const void* Wg, const void* Wu, int64_t T, int d, int G, int N, float* A_add,
@@ -396,7 +396,7 @@ int dtp_down_weight_sqnorm(const void* Wqkv_next, const void* gamma_next, const 
         return DTP_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DTP_CUDA_TRY(cudaMemsetAsync(workspace, 0, kWorkspaceHeader, s));
-    return sq::launch_down(Wqkv_next, gamma_next, W_down, H_kv, R, d, N, dtype, bn, workspace, s);
+    return sq::launch_down(Wqkv_next, gamma_next, W_down, H_kv, R, d, N, bn, workspace, s);
 }
 
 int dtp_down_finalize(const float* act2, const float* bn, int H_kv, int N, int64_t T_total, float* S_down,

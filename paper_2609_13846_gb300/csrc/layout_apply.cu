@@ -754,7 +754,7 @@ int launch_layout(const int32_t* head_part, const int32_t* neuron_dev, int layer
     if (g.n > 0) {
         const int grid = grid_for_rows(g.total, bytes / g.total);
         if (grid < 0) return DTP_ERR_CUDA;
-            gather_jobs_kernel<<<grid, 256, 0, stream>>>(g, status);
+        gather_jobs_kernel<<<grid, 256, 0, stream>>>(g, status);
         DTP_CUDA_TRY(cudaGetLastError());
     }
     for (int i = 0; i < 7; ++i) {

@@ -108,7 +108,7 @@ struct Shared {
     float scale[DMAX];                     // a device's mean gain in units of 2^sh (relative size only)
     int32_t price[DMAX];                   // prices in units of 2^sh, handed from one warp or block to the others
     int count[DMAX];
-    int64_t total, J, Jprev;
+    int64_t J, Jprev;
     int h[GMAX];
     int hn[GMAX];                          // next layer's head partition (whole-model search)
     int glist[GMAX], gnlist[GMAX];         // heads listed device by device, for h and for hn
@@ -498,8 +498,8 @@ struct Layer {
     int n, k0;          // neurons of this block's slice (in a step: of the gains) and the first one's index
     int np;             // column stride of hi and lo
     int rnp;            // row stride of qh and ql
-    int32_t* hi;        // [D][np] gains >> 15
-    uint16_t* lo;       // [D][np] gains' low 15 bits
+    int32_t* hi;        // [D][np] gains >> sh
+    uint16_t* lo;       // [D][np] gains' low sh bits
     uint8_t* nu;        // [np]
     uint16_t* lists;    // neurons of the slice by device [D][rnp]: over the block's own gains
     uint32_t* qh;
@@ -1133,7 +1133,9 @@ __device__ __forceinline__ int gap_pass(const Layer& layer, int n, int cap, Team
 #pragma unroll
         for (int l = 0; l < DT; ++l)
             if (l != a) {
-                m = fminf(m, __uint2float_rz(static_cast<uint32_t>(va - v[l])) * fminf(ia, inv[l]));
+                // the difference of two int32 needs 32 bits without a sign
+                const uint32_t gap32 = static_cast<uint32_t>(va) - static_cast<uint32_t>(v[l]);
+                m = fminf(m, __uint2float_rz(gap32) * fminf(ia, inv[l]));
                 if (v[l] > vb) vb = v[l], b = l;
             }
         const uint32_t e = __float_as_uint(m) >> 20;
@@ -1353,7 +1355,8 @@ __device__ __noinline__ void neuron_step_general(const Layer& L, Team& tm) {
             for (int l = 0; l < DT; ++l) hs[l] += static_cast<uint32_t>(hi_of<SM>(L)[l * L.np + k]) >> 10;
 #pragma unroll
         for (int l = 0; l < DT; ++l) {
-            const uint32_t s = __reduce_add_sync(0xFFFFFFFFu, hs[l]);
+            // below 2^19 a neuron: slices in shared memory stay within 32 bits, larger ones need not
+            const int64_t s = SM ? __reduce_add_sync(0xFFFFFFFFu, hs[l]) : warp_sum_i64(hs[l]);
             if (lane == 0) sh.part[warp][l] = s;
         }
         __syncthreads();

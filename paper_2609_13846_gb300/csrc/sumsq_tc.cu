@@ -566,12 +566,11 @@ size_t down_workspace_bytes(int G, int R, int d, int N) {
            static_cast<size_t>(units) * BCOL * sizeof(float);
 }
 
-int launch_down(const void* Wqkv, const void* gamma, const void* Wd, int G, int R, int d, int N, int dtype, float* bn,
+int launch_down(const void* Wqkv, const void* gamma, const void* Wd, int G, int R, int d, int N, float* bn,
                 void* workspace, cudaStream_t stream) {
     uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
     __nv_bfloat16* WdT = reinterpret_cast<__nv_bfloat16*>(ws + kWorkspaceHeader);
     float* partial = reinterpret_cast<float*>(ws + kWorkspaceHeader + align_up(static_cast<size_t>(N) * d * 2, 256));
-    if (dtype != DTP_BF16) return DTP_ERR_UNSUPPORTED;
     const bool wide = N % 8 == 0;                               // Wd is 16-byte aligned
     const int tile = wide ? kPrepTileOf<true> : kPrepTileOf<false>;
     const dim3 pg((N + tile - 1) / tile, (d + tile - 1) / tile);
