@@ -78,3 +78,14 @@ def test_add_and_down_edge_reject_host_tensors():
         dtp.down_weight_sqnorm(_bf16(2, 24, 64), _bf16(64), _bf16(64, 128))
     with pytest.raises(ValueError, match="CUDA"):
         dtp.down_finalize(torch.zeros(128), torch.zeros(2, 128), 16)
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_current_stream_with_and_without_the_raw_handle(monkeypatch, raw):
+    """The stream of a call is the current device's, also on a torch without the raw-handle function."""
+    from types import SimpleNamespace
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=77))
+    monkeypatch.setattr(dtp, "_current_raw_stream", (lambda index: 70 + index) if raw else None)
+    assert dtp._stream() == (73 if raw else 77)
+    assert dtp._stream(SimpleNamespace(cuda_stream=5)) == 5
