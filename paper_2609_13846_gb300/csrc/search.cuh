@@ -107,6 +107,8 @@ struct Shared {
     int64_t pi[DMAX];                      // device prices
     float scale[DMAX];                     // a device's mean gain in units of 2^sh (relative size only)
     int32_t price[DMAX];                   // prices in units of 2^sh, handed from one warp or block to the others
+    int32_t best_price[DMAX];              // the prices of the smallest excess so far
+    int32_t price_step[DMAX];              // the size of a price's last change by a sweep (negative: none yet)
     int count[DMAX];
     int64_t J, Jprev;
     int h[GMAX];
@@ -913,8 +915,8 @@ __device__ __noinline__ void exchange_graph(const Layer& L, Team& tm, int lo) {
     const int first = lo < L.k0 ? 0 : lo + 1 - L.k0;
     if (threadIdx.x < DMAX * DMAX) wl[threadIdx.x] = 0;
     __syncthreads();
-    for (int a = 0; a < DT; ++a) {
-        if (!((rows >> a) & 1u)) continue;
+    for (unsigned left = rows; left; left &= left - 1) {
+        const int a = __ffs(left) - 1;
         uint64_t best[DT];
 #pragma unroll
         for (int b = 0; b < DT; ++b) best[b] = 0;
@@ -947,14 +949,25 @@ __device__ __noinline__ void exchange_graph(const Layer& L, Team& tm, int lo) {
     tm.wph ^= 1;
 }
 
-// Lane b: the gains of the edges into device b of an exchange graph (kNegInf: none).
+// bellman_ford_warp on an exchange graph in shared memory: the edges stay there, as registers that this
+// takes are taken from the price steps.
 template <int DT>
-__device__ __forceinline__ void edges_into(const uint64_t (&graph)[DMAX][DMAX], int64_t (&w)[DT]) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int a = 0; a < DT; ++a) {
-        const uint64_t e = lane < DT && lane != a ? graph[a][lane] : 0;
-        w[a] = e ? gain_of(e) : kNegInf;
+__device__ __forceinline__ void bellman_ford_graph(const uint64_t (&graph)[DMAX][DMAX], unsigned src, int64_t& dist,
+                                                   int& pred) {
+    const int b = threadIdx.x & 31;
+    dist = (src >> b) & 1u ? 0 : kNegInf;
+    pred = -1;
+#pragma unroll 1
+    for (int round = 0; round < DT - 1; ++round) {
+        const int64_t before = dist;
+        bool moved = false;
+#pragma unroll 1
+        for (int a = 0; a < DT; ++a) {
+            const int64_t from = __shfl_sync(0xFFFFFFFFu, before, a);
+            const uint64_t e = b < DT && b != a ? graph[a][b] : 0;
+            if (e && from != kNegInf && from + gain_of(e) > dist) dist = from + gain_of(e), pred = a, moved = true;
+        }
+        if (!__any_sync(0xFFFFFFFFu, moved)) break;
     }
 }
 
@@ -981,6 +994,73 @@ __device__ __forceinline__ int apply_path(const Layer& L, const uint64_t (&graph
     return -1;
 }
 
+// Warp 0's parts of the repair, out of line: their registers would be taken from the price steps.
+// One unit of excess along the maximum-gain path of sh.w.
+template <int DT, bool SM>
+__device__ __noinline__ void move_excess(const Layer& L) {
+    Shared& sh = shared();
+    const int lane = threadIdx.x & 31;
+    const int cnt = lane < DT ? sh.count[lane] : L.cap;
+    const unsigned src = __ballot_sync(0xFFFFFFFFu, cnt > L.cap);
+    const unsigned snk = __ballot_sync(0xFFFFFFFFu, cnt < L.cap);
+    int64_t dist;
+    int pred;
+    bellman_ford_graph<DT>(sh.w, src, dist, pred);
+    int e = -1;
+    int64_t best = kNegInf;
+#pragma unroll 1
+    for (int b = 0; b < DT; ++b) {
+        const int64_t x = __shfl_sync(0xFFFFFFFFu, dist, b);
+        if (((snk >> b) & 1u) && x > best) best = x, e = b;
+    }
+    const int s = e < 0 ? -1 : apply_path<DT, SM>(L, sh.w, pred, e);
+    if (lane == 0) {
+        if (s < 0) sh.status = DTP_ERR_NOT_CONVERGED;
+        else sh.count[s] -= 1, sh.count[e] += 1;
+    }
+}
+
+// All-pairs paths of sh.w, and prices for the next neuron step: longest paths from a zero root.
+template <int DT>
+__device__ __noinline__ void close_graph() {
+    Shared& sh = shared();
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < DT * DT; i += 32) {
+        const int a = i / DT, b = i % DT;
+        sh.P[a][b] = a == b ? 0 : (sh.w[a][b] ? gain_of(sh.w[a][b]) : kNegInf);
+    }
+    __syncwarp();
+    close_paths(DT);
+    if (lane < DT) {
+        if (sh.P[lane][lane] > 0) sh.status = DTP_ERR_NOT_CONVERGED;   // a positive cycle: not optimal
+        int64_t pot = 0;
+        for (int a = 0; a < DT; ++a) pot = sh.P[a][lane] > pot ? sh.P[a][lane] : pot;
+        sh.pi[lane] = pot;
+    }
+}
+
+// Neuron kstar (its gains and its device t in sh.B) to the smallest device that a zero-gain path through
+// sh.wk back to t allows.
+template <int DT, bool SM>
+__device__ __noinline__ void move_earlier(const Layer& L, int kstar) {
+    Shared& sh = shared();
+    const int lane = threadIdx.x & 31;
+    const int t = static_cast<int>(sh.B[DT]);
+    int64_t dist;
+    int pred;
+    if (lane == 0) sh.dirty = 0;
+#pragma unroll 1
+    for (int l = 0; l < t; ++l) {
+        bellman_ford_graph<DT>(sh.wk, 1u << l, dist, pred);
+        const int64_t to = __shfl_sync(0xFFFFFFFFu, dist, t);
+        if (to == kNegInf || sh.B[l] - sh.B[t] + to != 0) continue;
+        if (apply_path<DT, SM>(L, sh.wk, pred, t) < 0 && lane == 0) sh.status = DTP_ERR_NOT_CONVERGED;
+        const int k = kstar - L.k0;
+        if (lane == 0 && k >= 0 && k < L.n) nu_of<SM>(L)[k] = static_cast<uint8_t>(l);
+        break;
+    }
+}
+
 // Step (d) over all neurons.  assigned: L.nu is already optimal; else it is the assignment at some
 // prices and is balanced first.  Warp 0 of every block of a team repeats the steps over the devices on
 // equal data.
@@ -988,7 +1068,6 @@ template <int DT, bool SM>
 __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned) {
     Shared& sh = shared();
     const int N = L.N, D = L.D, cap = L.cap;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) sh.dirty = (1u << DT) - 1u;
     __syncthreads();
     if (!assigned) {
@@ -1002,27 +1081,8 @@ __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned)
             for (int l = 0; l < D; ++l) ex += sh.count[l] > cap ? 1 : 0;
             if (ex == 0) break;
             exchange_graph<DT, SM>(L, tm, -1);
-            if (warp == 0) {
-                if (lane == 0 && sh.beat && (aug & 31) == 31) atomicAdd(sh.beat, 1);
-                const int cnt = lane < DT ? sh.count[lane] : cap;
-                const unsigned src = __ballot_sync(0xFFFFFFFFu, cnt > cap);
-                const unsigned snk = __ballot_sync(0xFFFFFFFFu, cnt < cap);
-                int64_t w[DT], dist;
-                int pred;
-                edges_into<DT>(sh.w, w);
-                bellman_ford_warp<DT>(src, w, dist, pred);
-                int e = -1;
-                int64_t best = kNegInf;
-                for (int b = 0; b < DT; ++b) {
-                    const int64_t x = __shfl_sync(0xFFFFFFFFu, dist, b);
-                    if (((snk >> b) & 1u) && x > best) best = x, e = b;
-                }
-                const int s = e < 0 ? -1 : apply_path<DT, SM>(L, sh.w, pred, e);
-                if (lane == 0) {
-                    if (s < 0) sh.status = DTP_ERR_NOT_CONVERGED;
-                    else sh.count[s] -= 1, sh.count[e] += 1;
-                }
-            }
+            if (threadIdx.x < 32) move_excess<DT, SM>(L);
+            if (threadIdx.x == 0 && sh.beat && (aug & 31) == 31) atomicAdd(sh.beat, 1);
             __syncthreads();
             if (sh.status != DTP_OK) return;
         }
@@ -1037,22 +1097,8 @@ __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned)
     int kstart = 0;
     for (int round = 0; round < N + 1; ++round) {
         exchange_graph<DT, SM>(L, tm, -1);
-        if (warp == 0) {
-            if (lane == 0 && sh.beat && (round & 31) == 31) atomicAdd(sh.beat, 1);
-            for (int i = lane; i < DT * DT; i += 32) {
-                const int a = i / DT, b = i % DT;
-                sh.P[a][b] = a == b ? 0 : (sh.w[a][b] ? gain_of(sh.w[a][b]) : kNegInf);
-            }
-            __syncwarp();
-            close_paths(DT);
-            if (lane < DT) {
-                if (sh.P[lane][lane] > 0) sh.status = DTP_ERR_NOT_CONVERGED;   // a positive cycle: not optimal
-                // prices for the next neuron step: longest paths from a zero root
-                int64_t pot = 0;
-                for (int a = 0; a < DT; ++a) pot = sh.P[a][lane] > pot ? sh.P[a][lane] : pot;
-                sh.pi[lane] = pot;
-            }
-        }
+        if (threadIdx.x < 32) close_graph<DT>();
+        if (threadIdx.x == 0 && sh.beat && (round & 31) == 31) atomicAdd(sh.beat, 1);
         __syncthreads();
         if (sh.status != DTP_OK) return;
         uint32_t cand = static_cast<uint32_t>(N);
@@ -1079,22 +1125,7 @@ __device__ __noinline__ void repair_all(const Layer& L, Team& tm, bool assigned)
                 !own ? 0 : (threadIdx.x < DT ? gain_at<SM>(L, threadIdx.x, k) : static_cast<int64_t>(nu_of<SM>(L)[k]));
         }
         team_sum_i64(DT + 1, tm);
-        if (warp == 0) {
-            const int t = static_cast<int>(sh.B[DT]);
-            int64_t w[DT], dist;
-            int pred;
-            edges_into<DT>(sh.wk, w);
-            if (lane == 0) sh.dirty = 0;
-            for (int l = 0; l < t; ++l) {
-                bellman_ford_warp<DT>(1u << l, w, dist, pred);
-                const int64_t to = __shfl_sync(0xFFFFFFFFu, dist, t);
-                if (to == kNegInf || sh.B[l] - sh.B[t] + to != 0) continue;
-                if (apply_path<DT, SM>(L, sh.wk, pred, t) < 0 && lane == 0) sh.status = DTP_ERR_NOT_CONVERGED;
-                const int k = kstar - L.k0;
-                if (lane == 0 && k >= 0 && k < L.n) nu_of<SM>(L)[k] = static_cast<uint8_t>(l);
-                break;
-            }
-        }
+        if (threadIdx.x < 32) move_earlier<DT, SM>(L, kstar);
         __syncthreads();
         if (sh.status != DTP_OK) return;
         kstart = kstar + 1;
@@ -1212,12 +1243,12 @@ __device__ __forceinline__ void newton_step(int cap, float tau, int32_t (&p)[DT]
 }
 
 // A Gauss-Seidel sweep over n neurons of a slice: each price in turn is set so that about cap neurons
-// (within tol) prefer its device at the others' prices.  step[l]: the size of price l's last change
-// (negative: none yet); a histogram of the keys around the old price on that scale usually holds the
-// new one, which saves the pass for their range and the refinement.
+// (within tol) prefer its device at the others' prices.  A histogram of the keys around the old price on
+// the scale of its last change (sh.price_step: every thread would keep the same) usually holds the new
+// one, which saves the pass for their range and the refinement.
 template <int DT, bool SM>
 __device__ __forceinline__ void price_sweep(const Layer& layer, int n, int cap, uint32_t tol, Team& tm,
-                                         int32_t (&prices)[DT], int32_t (&step)[DT]) {
+                                         int32_t (&prices)[DT]) {
     Shared& sh = shared();
     const Layer L = layer;
     int32_t p[DT];
@@ -1236,10 +1267,11 @@ __device__ __forceinline__ void price_sweep(const Layer& layer, int n, int cap, 
             x = static_cast<uint32_t>(own - alt) ^ 0x80000000u;
             return true;
         };
-        int32_t old = 0, width = -1;
+        int32_t old = 0;
 #pragma unroll
         for (int m = 0; m < DT; ++m)
-            if (m == l) old = p[m], width = step[m];
+            if (m == l) old = p[m];
+        const int32_t width = sh.price_step[l];
         uint32_t t = 0, ge = 0;
         bool found = false;
         if (width >= 0) {
@@ -1279,7 +1311,7 @@ __device__ __forceinline__ void price_sweep(const Layer& layer, int n, int cap, 
             if (m == l) {
                 const int64_t d = static_cast<int64_t>(now) - p[m];
                 const int64_t ad = d < 0 ? -d : d;
-                step[m] = static_cast<int32_t>(ad < kPriceMax / 4 ? ad : kPriceMax / 4);
+                if (threadIdx.x == 0) sh.price_step[m] = static_cast<int32_t>(ad < kPriceMax / 4 ? ad : kPriceMax / 4);
                 p[m] = now;
             }
     }
@@ -1297,9 +1329,7 @@ template <int DT, bool SM>
 __device__ __noinline__ float find_prices(const Layer& L, int n, int cap, int stop, int most, Team& tm,
                                           int32_t (&p)[DT]) {
     Shared& sh = shared();
-    int32_t best_p[DT], step[DT];
-#pragma unroll
-    for (int l = 0; l < DT; ++l) step[l] = -1;
+    if (threadIdx.x < DT) sh.price_step[threadIdx.x] = -1;      // read after the first gap_pass's barriers
     int best = INT32_MAX, stalled = 0;
     bool newton = false;
     float tau = 0.015625f;
@@ -1313,16 +1343,17 @@ __device__ __noinline__ float find_prices(const Layer& L, int n, int cap, int st
             if (!newton) stalled = 0;
             best = excess;
 #pragma unroll
-            for (int l = 0; l < DT; ++l) best_p[l] = p[l];
+            for (int l = 0; l < DT; ++l)
+                if (threadIdx.x == 0) sh.best_price[l] = p[l];   // read after the next gap_pass's barriers
         } else {
             if (!newton) ++stalled;                  // ties: no price separates them
 #pragma unroll
-            for (int l = 0; l < DT; ++l) p[l] = best_p[l];
+            for (int l = 0; l < DT; ++l) p[l] = sh.best_price[l];
             sweep = true;
         }
         newton = !sweep && best <= cap * DT / 12;
         if (newton) newton_step<DT>(cap, tau, p);
-        else price_sweep<DT, SM>(L, n, cap, static_cast<uint32_t>(best / (4 * DT)) + 1u, tm, p, step);
+        else price_sweep<DT, SM>(L, n, cap, static_cast<uint32_t>(best / (4 * DT)) + 1u, tm, p);
         // pairs are counted next time within twice the gap that holds the nearest candidates
         if (gap.found && gap.above > 0) tau = 2.0f * __uint_as_float(gap.bin);
     }
@@ -1330,8 +1361,9 @@ __device__ __noinline__ float find_prices(const Layer& L, int n, int cap, int st
     return gap.above == 0 ? 0.0f : __uint_as_float(gap.bin);
 }
 
+// Steps (a) to (c).  Returns what repair_all still has to do: 0 nothing, 1 the lexicographic order, 2 all.
 template <int DT, bool SM>
-__device__ __noinline__ void neuron_step_general(const Layer& L, Team& tm) {
+__device__ __noinline__ int neuron_step_general(const Layer& L, Team& tm) {
     Shared& sh = shared();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int32_t p[DT];                       // prices, the same in every thread of the team
@@ -1396,20 +1428,17 @@ __device__ __noinline__ void neuron_step_general(const Layer& L, Team& tm) {
         }
         tau = find_prices<DT, SM>(L, L.n, L.cap, stop, any, tm, p);
     }
-    // (b), (c), and (d) where they give no certificate
+    // (b) and (c)
     bool unique;
-    if (assign_candidates<DT, SM>(L, tm, p, tau, unique)) {
-        if (!unique) repair_all<DT, SM>(L, tm, true);
-    } else {
-        repair_all<DT, SM>(L, tm, false);
-    }
+    if (!assign_candidates<DT, SM>(L, tm, p, tau, unique)) return 2;
+    return unique ? 0 : 1;
 }
 
 template <int DT, bool SM>
 __device__ __forceinline__ void neuron_step(const Layer& L, Team& tm) {
     Shared& sh = shared();
     if constexpr (DT == 2) neuron_step_d2<SM>(L, tm);
-    else neuron_step_general<DT, SM>(L, tm);
+    else if (const int left = neuron_step_general<DT, SM>(L, tm)) repair_all<DT, SM>(L, tm, left == 1);   // (d)
 }
 
 // --------------------------------------------------------------- head step --
