@@ -544,9 +544,9 @@ def main():
     stream = torch.cuda.current_stream()
     side = torch.cuda.Stream(device=dev)
     n_sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    # Step pipeline: the affinity pass of step k runs on all SMs but one (max_ctas; for this layer
-    # its CTA pairs round that down to 150 of 152) while the layout search of step k-1 (one thread
-    # block) runs on a spare SM from a second stream.
+    # Step pipeline: the affinity pass of step k is capped one CTA below the chip (max_ctas; the library
+    # rounds that down to an even count, 150 of 152) while the layout search of step k-1 (a cluster of
+    # two thread blocks) runs on the two SMs left, from a second stream.
     # A and the search workspace are double-buffered; events order each buffer's reuse.  (Moving
     # the 12 us partial-sum reduce to the second stream as well measured slower.)
     A_buf = [torch.zeros((w.G, w.N), dtype=torch.float32, device=dev) for _ in range(2)]
@@ -847,8 +847,8 @@ def main():
         "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
         "config": {"workload": WORKLOAD, "d": w.d, "G": w.G, "N": w.N, "T": w.T, "D": D, "iters": iters,
                    "layers_per_step": world, "l2": "inputs (302 MB) larger than L2; no flush",
-                   "pipeline": "two streams: step k's affinity on all SMs but one, step k-1's search on the "
-                               "spare SM; A double-buffered"},
+                   "pipeline": "two streams: step k's affinity on all SMs but two, step k-1's search on "
+                               "those two; A double-buffered"},
         "affinity_ms": aff_mean_ms, "affinity_tflops": achieved, "search_ms": search_ms,
         "search_iters_done": int(res["iters_done"]), "layout_score": float(res["score"]),
         "model_search": model_search,

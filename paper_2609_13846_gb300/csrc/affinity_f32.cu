@@ -28,7 +28,8 @@ constexpr int kTokMin = 64;   // tokens per tile of the smaller form (the worksp
 // the loads the limit; 4 x 4 (64 x 64 tiles, two blocks per SM) for layers with few tiles.  alpha and beta
 // live in shared memory, the next k block is loaded from global memory during the current one.
 // T = 1024, d = 1024, 8 heads, N = 3072 on a GB300: 4.34 ms with 4 x 4 scalar tiles, 2.80 ms with 8 x 4
-// packed ones (FMA pipe 62% busy, shared wavefronts 63%), 2.40 with 8 x 8 (70%).
+// packed ones, 2.40 with 8 x 8.  There the FMA pipe is 70% busy and the shared-memory path 57%: with two
+// warps a scheduler the rest is waiting at barriers, for shared loads and in the epilogues.
 template <int TPT, int NPT>
 struct Tile {
     static constexpr int TM = 16 * TPT;          // tokens
