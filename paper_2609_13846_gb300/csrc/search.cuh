@@ -1446,8 +1446,10 @@ __device__ __forceinline__ void neuron_step(const Layer& L, Team& tm) {
 // sh.xl[phase][r * DT + l] = the slice's sum of score row r over its neurons on device l, for rows
 // r < rows; nu: the slice's labels.  The neurons are first listed by device (over the gains, which the
 // next step rebuilds),
-// then a power of two of threads adds each (row, device) list (several warps where there are few
-// lists): 2.5 times fewer instructions than walking every row with a select per device.
+// then a power of two of threads adds each (row, device) list: 2.5 times fewer instructions than
+// walking every row with a select per device.  In global memory, where the loads' latency counts, several
+// warps add a list where there are few, four neurons at a time; in shared memory that would only be more code
+// to fetch (1 us of a small layer's 25).
 template <int DT, bool SM>
 __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, Team& tm, int rows) {
     Shared& sh = shared();
@@ -1457,7 +1459,7 @@ __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, 
     const bool wide = L.rnp > 65535;            // 32-bit indices: only where no cluster of four can be resident
     uint32_t* lists32 = reinterpret_cast<uint32_t*>(lists);
     if (tid < DMAX) sh.clen[tid] = 0;
-    if (tid < rows * DT) sh.xl[tm.lph][tid] = 0;
+    if (!SM && tid < rows * DT) sh.xl[tm.lph][tid] = 0;
     __syncthreads();
     for (int k0 = 0; k0 < L.n; k0 += kThreads) {
         const int k = k0 + tid;
@@ -1473,8 +1475,8 @@ __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, 
     }
     __syncthreads();
     const int pairs = rows * DT;                                // 4 to 256
-    int tpp = kThreads / 4;
-    while (tpp * pairs > kThreads) tpp >>= 1;                   // 2 to 128
+    int tpp = SM ? 32 : kThreads / 4;
+    while (tpp * pairs > kThreads) tpp >>= 1;                   // from 2
     if (tid < pairs * tpp) {                                    // whole groups of tpp lanes, or whole warps
         const int pair = tid / tpp, sub = tid % tpp;
         const int r = pair / DT, l = pair % DT;
@@ -1485,15 +1487,17 @@ __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, 
             return wide ? static_cast<int>(lists32[l * L.rnp + j]) : lists[l * L.rnp + j];
         };
         int j = sub;
-        for (; j + 3 * tpp < len; j += 4 * tpp) {               // four neurons' loads in flight
-            int k[4];
-            uint32_t h[4], lo[4];
+        if constexpr (!SM) {
+            for (; j + 3 * tpp < len; j += 4 * tpp) {           // four neurons' loads in flight
+                int k[4];
+                uint32_t h[4], lo[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) k[u] = entry(j + u * tpp);
+                for (int u = 0; u < 4; ++u) k[u] = entry(j + u * tpp);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) score_parts<SM>(L, r, k[u], h[u], lo[u]);
+                for (int u = 0; u < 4; ++u) score_parts<SM>(L, r, k[u], h[u], lo[u]);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) hs += h[u], ls += lo[u];
+                for (int u = 0; u < 4; ++u) hs += h[u], ls += lo[u];
+            }
         }
         for (; j < len; j += tpp) {
             uint32_t h, lo;
@@ -1506,7 +1510,7 @@ __device__ __noinline__ void column_sums(const Layer& layer, const uint8_t* nu, 
         const unsigned group = (0xFFFFFFFFu >> (32 - width)) << (lane & ~(width - 1));
         int64_t v = (hs << kLoBits) + ls;
         for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(group, v, o);
-        if (tpp <= 32) {
+        if (SM || tpp <= 32) {
             if (sub == 0) sh.xl[tm.lph][pair] = v;
         } else if (lane == 0) {
             atomicAdd(reinterpret_cast<unsigned long long*>(&sh.xl[tm.lph][pair]), static_cast<unsigned long long>(v));
